@@ -27,6 +27,7 @@
 #include <unordered_map>
 
 #include "device_util.cuh"
+#include "ext_view.cuh"
 #include "kernels.h"
 #include "state.h"
 #include "tc_ptx.cuh"
@@ -153,7 +154,6 @@ __global__ void __launch_bounds__(128) k_begin(Config cfg) {
 // grid = (tiles^2, walkers * 2), block 256, dynamic shared memory.
 // ---------------------------------------------------------------------------
 constexpr int TT = 32;   // tile of the update kernel
-constexpr int METRO_SMEM_KS = 96;  // largest k_s whose B^-1 (both spins) lives in shared memory
 constexpr int ET = 64;   // tile of the extension kernel
 constexpr int EC = 32;   // candidates per pass
 
@@ -448,57 +448,6 @@ __global__ void __launch_bounds__(256, sizeof(A) == 4 ? 3 : 2) k_cand_cc(Config 
 // ---------------------------------------------------------------------------
 // Metropolis over the window (one block per walker, both spins).
 // ---------------------------------------------------------------------------
-template <typename T>
-struct ExtView {
-  const T* N;        // current N (ld)
-  const T* X;        // candidate rows [c][ld] (stored like N)
-  const double* Gc;  // candidate columns [c][ld]
-  const int* vs;
-  int n, ld;
-};
-
-template <typename T>
-__device__ __forceinline__ ExtView<T> make_view(const WalkerDev& w, int sp) {
-  ExtView<T> v;
-  v.N = (const T*)w.N[w.parity][sp];
-  v.X = reinterpret_cast<const T*>(w.Xr[sp]);
-  v.Gc = w.Gc[sp];
-  v.vs = w.vs[w.parity];
-  v.n = w.n;
-  v.ld = w.cap;
-  return v;
-}
-
-// G_ext[x, y]; for an interacting existing column y, G = (N e^{V} - I) / (e^{V} - 1)
-// column-wise, which follows from N = [I + G (e^V - I)] e^{-V}.
-template <typename T>
-__device__ __forceinline__ double g_ext(const ExtView<T>& v, const ProblemDev& pb, int sp, int x, int y) {
-  if (y >= v.n) return v.Gc[(size_t)(y - v.n) * v.ld + x];
-  const double nxy = ldN(x < v.n ? v.N : v.X, (size_t)(x < v.n ? x : x - v.n) * v.ld + y);
-  const int sy = v.vs[y];
-  const double ev = expV(pb, sp, sy);
-  // (N e^V - 1) / (e^V - 1) with the reciprocal tabulated per spin (no FP64 division)
-  return (nxy * ev - (x == y ? 1.0 : 0.0)) * pb.rexpVm1[sp][sy > 0 ? 1 : 0];
-}
-
-// G_ext[x, y] with the spin factors of column y given: e^{V_y} and
-// 1 / (e^{V_y} - 1) (unused for a candidate column y >= n).
-template <typename T>
-__device__ __forceinline__ double g_ext_at(const ExtView<T>& v, int x, int y, double ev, double rv) {
-  if (y >= v.n) return v.Gc[(size_t)(y - v.n) * v.ld + x];
-  const double nxy = ldN(x < v.n ? v.N : v.X, (size_t)(x < v.n ? x : x - v.n) * v.ld + y);
-  return (nxy * ev - (x == y ? 1.0 : 0.0)) * rv;
-}
-
-// Address of the stored entry g_ext_at reads for (x, y).
-template <typename T>
-__device__ __forceinline__ const void* g_ext_ptr(const ExtView<T>& v, int x, int y) {
-  if (y >= v.n) return v.Gc + (size_t)(y - v.n) * v.ld + x;
-  return (x < v.n) ? (const void*)(v.N + (size_t)x * v.ld + y) : (const void*)(v.X + (size_t)(x - v.n) * v.ld + y);
-}
-
-__device__ __forceinline__ void prefetch_l1(const void* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
-
 // Arithmetic M of the bordered growth of B^-1 and of the Schur complements
 // (the determinant ratios): FP64 (double), or double-float pairs (hi, lo) of
 // FP32 (float2), about 44 significant bits at the FP32 issue rate.  The
@@ -541,8 +490,8 @@ __device__ __forceinline__ int row_lanes(int l) {
   return G;
 }
 
-constexpr int METRO_LIVE = 2048;  // live vertices whose rows and spins are staged in shared memory
-
+// Metropolis with Gamma in double-float pairs (DCA_GAMMA_DOUBLE_FLOAT; FP64 Gamma
+// runs in k_metropolis.cu).
 // One block per walker, both spins.  Per proposal: (1) its target and a_t,
 // (2) the border of B against the accepted set P, (3) t = B^-1 b_col, (4) the
 // Schur complements d_sigma = B_tt - b_row t, (5) the decision on
@@ -1030,62 +979,7 @@ __global__ void __launch_bounds__(256) k_metropolis(Config cfg) {
         w.vs[w.parity][s_P[p]] = s_Pup[p] ? 1 : -1;  // its spin (a flip in the window may have changed it)
         ++m;
       }
-    const int eval = s_eval;
-    w.n_acc = l;
-    w.n_removed = nrem;
-    w.n_ins = nins;
-    w.n_eval = eval;
-    w.aborted = (eval < len) && w.status == ST_OK;
-    w.sign = s_sign;
-    if (w.status == ST_OK) {
-      w.q += (uint64_t)eval;
-      w.sweep_pos += eval;
-      w.n_windows++;
-      if (w.aborted) w.n_aborts++;
-      const int64_t sweep_no = w.sweeps_done;  // the sweep this window belongs to
-      if (w.sweep_pos >= w.sweep_len_cur) {
-        w.measure_pending = (w.sweeps_done >= cfg.warmup) ? 1 : 0;
-        w.sweeps_done++;
-        w.sweep_pos = 0;
-      }
-      w.windows_since_recompute++;
-      if (cfg.recompute_every > 0 && w.windows_since_recompute >= cfg.recompute_every) {
-        w.recompute_pending = 1;
-        w.windows_since_recompute = 0;
-      }
-      // Batched schedule: every walker recomputes after the first window of
-      // every recompute_sweeps-th sweep (the same window for all walkers).
-      // (With N recomputed at every measurement the measured sweeps need no other.)
-      if (cfg.recompute_sweeps > 0 && w.first_window && sweep_no > 0 && sweep_no % cfg.recompute_sweeps == 0 &&
-          !(cfg.recompute_at_measure && sweep_no > cfg.warmup)) {
-        w.recompute_pending = 1;
-        w.windows_since_recompute = 0;
-      }
-      // Fresh N for every measurement: the recompute runs in the window that
-      // ends the sweep, before the measurement.
-      if (cfg.recompute_at_measure && w.measure_pending) {
-        w.recompute_pending = 1;
-        w.windows_since_recompute = 0;
-      }
-      // Algorithmic work per spin on the k live vertices after the window:
-      // update 2 k^2 l + 2 k l^2 flop, reading and writing k^2 entries of N
-      // plus the k x l factors; extension 4 k0^2 c flop and one read of N (both
-      // candidate products need only that one read).
-      const double b = cfg.prec == PREC_MIXED ? 4.0 : 8.0;
-      const double kk = (double)(n_live - nrem + nins), ll = (double)l;
-      if (l > 0) {
-        w.flops += 2.0 * (2.0 * kk * kk * ll + 2.0 * kk * ll * ll);
-        w.upd_bytes += 2.0 * (b * 2.0 * kk * kk + 8.0 * 2.0 * kk * ll);
-      }
-      const double k0 = (double)n_live, cc = (double)w.n_cand;
-      if (w.n_cand > 0) {
-        w.ext_flops += 2.0 * (4.0 * k0 * k0 * cc);
-        w.ext_bytes += 2.0 * b * (k0 * k0);
-      }
-    } else {
-      w.active = 0;
-      w.n_acc = 0;
-    }
+    metro_finish(cfg, w, n_live, len, l, nrem, nins, s_eval, s_sign);
   }
 }
 
@@ -1601,9 +1495,12 @@ static int launch_group_t(int group, const Config& cfg, int max_cap, cudaStream_
       k_cand_cc<A><<<grid_for(S * 16), 256, 0, st>>>(cfg);
       return 3;
     case GROUP_METROPOLIS: {
-      const int sm = cfg.ks <= METRO_SMEM_KS ? (int)sizeof(double) * 2 * cfg.ks * (cfg.ks | 1) : 0;
-      if (sizeof(T) == 8 || cfg.gamma_fp64) k_metropolis<T, double><<<W, 256, sm, st>>>(cfg);
-      else k_metropolis<T, float2><<<W, 256, sm, st>>>(cfg);
+      if (sizeof(T) == 8 || cfg.gamma_fp64) {
+        launch_metropolis64(cfg, st);
+      } else {
+        const int sm = cfg.ks <= METRO_SMEM_KS ? (int)sizeof(double) * 2 * cfg.ks * (cfg.ks | 1) : 0;
+        k_metropolis<float, float2><<<W, 256, sm, st>>>(cfg);
+      }
       return 1;
     }
     case GROUP_UPDATE_PRE:
@@ -1639,10 +1536,7 @@ cudaError_t setup_window_kernels() {
     e = cudaFuncSetAttribute(k_cand_ext<float, float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              ext_smem_bytes<float>());
   const int msm = (int)sizeof(double) * 2 * METRO_SMEM_KS * (METRO_SMEM_KS | 1);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_metropolis<double, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, msm);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_metropolis<float, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, msm);
+  if (e == cudaSuccess) e = setup_metropolis64();
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_metropolis<float, float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, msm);
   return e;

@@ -38,6 +38,10 @@ inline bool is_recompute_group(int g) {
 // and device before any launch or stream capture.
 cudaError_t setup_window_kernels();
 
+// Metropolis with FP64 Gamma (k_metropolis.cu).
+cudaError_t setup_metropolis64();
+void launch_metropolis64(const Config& cfg, cudaStream_t st);
+
 // Each launcher returns the number of kernels it launched.
 int launch_window_group(int group, const Config& cfg, int max_cap, cudaStream_t st);
 void launch_count_active(const Config& cfg, cudaStream_t st);
