@@ -93,6 +93,7 @@ struct dca_walker {
   int prec_public = 0;               // DCA_PREC_* given at create
   double* d_Mout = nullptr;          // read-out of the frequency measurement, all walkers
   long long* d_Mbase = nullptr;      // its per-walker offsets
+  double2* d_Mtab = nullptr;         // phases of the NFFT read-out
   double* d_Gout = nullptr;          // read-out of the tau-grid measurement, all walkers back to back
   long long* d_Gbase = nullptr;      // its per-walker offsets (gacc_off)
   double* h_Gout = nullptr;          // pinned host copy of d_Gout (one device-to-host copy per read-out)
@@ -1050,11 +1051,14 @@ extern "C" DCA_API int dca_walker_measure_M(dca_walker* h, double* M_out, double
     if (!h->d_Mout) {
       h->d_Mout = (double*)h->dalloc(sizeof(double) * total);
       h->d_Mbase = (long long*)h->dalloc(sizeof(long long) * h->W);
-      if (!h->d_Mout || !h->d_Mbase) return fail(h, DCA_ERR_OOM, "read-out buffers of the frequency measurement");
+      h->d_Mtab = (double2*)h->dalloc(sizeof(double2) * 2 * (size_t)h->cfg.nfft_L);
+      if (!h->d_Mout || !h->d_Mbase || !h->d_Mtab)
+        return fail(h, DCA_ERR_OOM, "read-out buffers of the frequency measurement");
       CK(cudaMemcpyAsync(h->d_Mbase, base.data(), sizeof(long long) * h->W, cudaMemcpyHostToDevice, h->stream));
+      dca::launch_nfft_table(h->cfg, h->d_Mtab, h->stream);
     }
     if (h->cfg.freq_dft) dca::launch_ndft_copy(h->cfg, h->max_nc, h->d_Mbase, h->d_Mout, h->stream);
-    else dca::launch_nfft_finish(h->cfg, h->max_nc, h->d_Mbase, h->d_Mout, h->stream);
+    else dca::launch_nfft_finish(h->cfg, h->max_nc, h->d_Mtab, h->d_Mbase, h->d_Mout, h->stream);
     h->total_launches += 1;
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(M_out, h->d_Mout, sizeof(double) * total, cudaMemcpyDeviceToHost, h->stream));
