@@ -231,7 +231,7 @@ def g4_assemble(A, D, sign_sum, G0_up, G0_dn):
     rc = L.dca_g4_assemble(int(S), _ptr(a), _ptr(d), float(sign_sum), _ptr(gu), _ptr(gd), _ptr(out))
     if rc != DCA_OK:
         raise WalkerError(rc, L.dca_walker_last_error(None).decode())
-    return out[..., 0] + 1j * out[..., 1]
+    return _from2(out)
 
 
 def _vertices(site, tau, s):
@@ -418,7 +418,7 @@ class Walkers:
         for nc in self.nc:
             k = 2 * nc * self.n_omega_meas * 2
             a = m[off:off + k].reshape(2, nc, self.n_omega_meas, 2)
-            out.append(a[..., 0] + 1j * a[..., 1])
+            out.append(_from2(a))
             off += k
         return out, ss, nm
 
@@ -435,7 +435,7 @@ class Walkers:
         for S in sizes:
             a = A[oa:oa + 2 * S * S].reshape(S, S, 2)
             d = D[od:od + 4 * S].reshape(2, S, 2)
-            out.append((a[..., 0] + 1j * a[..., 1], d[..., 0] + 1j * d[..., 1]))
+            out.append((_from2(a), _from2(d)))
             oa += 2 * S * S
             od += 4 * S
         return out, ss, nm
@@ -540,12 +540,14 @@ def _lattice(nc, kpts, k_dot_r, recip, t, tp, mu, U, beta, n_fine, keep):
 
 
 def _c2(a):
-    a = np.ascontiguousarray(a, np.complex128)
-    return np.ascontiguousarray(np.stack([a.real, a.imag], axis=-1))
+    """[..., re, im] view of a complex array (complex128 is stored as such pairs)."""
+    a = np.asarray(a, np.complex128, order="C")
+    return a.view(np.float64).reshape(a.shape + (2,))
 
 
 def _from2(a):
-    return a[..., 0] + 1j * a[..., 1]
+    """Complex view of a [..., re, im] array."""
+    return a.view(np.complex128)[..., 0]
 
 
 class DCALoop:
