@@ -53,8 +53,8 @@ constexpr size_t kOffSpin = kOffTau + up256(sizeof(double) * kMaxOrder);
 constexpr size_t kOffN0 = kOffSpin + up256(sizeof(int32_t) * kMaxOrder);
 constexpr size_t kOffN1 = kOffN0 + up256(sizeof(double) * kMaxOrder * kMaxOrder);
 constexpr size_t kOffScr0 = kOffN1 + up256(sizeof(double) * kMaxOrder * kMaxOrder);
-constexpr size_t kOffScr1 = kOffScr0 + up256(sizeof(double) * 2 * kMaxOrder);
-constexpr size_t kOffSign = kOffScr1 + up256(sizeof(double) * 2 * kMaxOrder);
+constexpr size_t kOffScr1 = kOffScr0 + up256(sizeof(double) * 16 * kMaxOrder);
+constexpr size_t kOffSign = kOffScr1 + up256(sizeof(double) * 16 * kMaxOrder);
 constexpr size_t kScratchBytes = kOffSign + up256(sizeof(int32_t) * 4);  // two signs, work queue
 
 static __device__ __align__(256) unsigned char g_fresh_scratch[kScratchBytes];
