@@ -5,7 +5,7 @@
 //   k_ext_x   X[c, j]         = sum_i U[c, i] N[i, j],   U[c, i] = g0(r_c - r_i, tau_c - tau_i) (e^{V_i} - 1)
 // V and U are the FP32 tables written by k_cand_zero (zero on dead vertices,
 // whose rows and columns therefore drop out).  The FP64 path keeps the tiled
-// one-pass kernel k_cand_ext.
+// kernels in k_extend64.cu.
 #include <cstdint>
 
 #include "device_util.cuh"

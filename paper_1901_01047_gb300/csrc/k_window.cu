@@ -3,10 +3,10 @@
 // Sequence per window (DCA++ paper Sec. 2.3, "Submatrix updates"):
 //   k_begin       proposals of the window from Philox (counter tag 0 / 1);
 //                 insertion candidates appended as non-interacting rows n + c
-//   k_cand_ext    one pass over N for both candidate products:
-//                 G_ext[i, n+c] = sum_j N[i,j] g0(r_j - r_c, tau_j - tau_c)
+//   k_cand_zero   the factors of both candidate products, tabulated
+//   k_ext*        G_ext[i, n+c] = sum_j N[i,j] g0(r_j - r_c, tau_j - tau_c)
 //                 X[c, j]     = sum_i g0(r_c - r_i, tau_c - tau_i) (e^{V_i} - 1) N[i,j]
-//   k_cand_cc     G_ext[n+c', n+c] = X[c',:] . g0[:, c] + g0(c', c)
+//   k_cc64, k_cand_cc  G_ext[n+c', n+c] = X[c',:] . g0[:, c] + g0(c', c)
 //   k_metropolis  serial single-spin decisions from B_P^-1 (bordered growth)
 //   k_upd_*       N <- N + (G[:,P] - E_P) diag(a_P) B^-1 N[P,:]: in place on
 //                 rows / columns 0..n-1, plus the rows and columns of the
@@ -143,59 +143,61 @@ __global__ void __launch_bounds__(128) k_begin(Config cfg) {
   }
 }
 
-// ---------------------------------------------------------------------------
-// Candidate extension, both products in one pass over N (SIMT).  A 64 x 64
-// tile N[I, J] contributes
-//   G_ext[I, n+c] += N[I, J] V[J, c],  V[j, c] = g0(r_j - r_c, tau_j - tau_c)
-//   X[c, J]       += U[c, I] N[I, J],  U[c, i] = g0(r_c - r_i, tau_c - tau_i) (e^{V_i} - 1)
-// and the partial sums are reduced into the FP64 buffers Gc / Xr with
-// atomics (zeroed by k_cand_zero).  Dead rows have e^V - 1 = 0 and dead
-// columns of N are unit columns, so both are skipped.
-// grid = (tiles^2, walkers * 2), block 256, dynamic shared memory.
-// ---------------------------------------------------------------------------
-constexpr int TT = 32;   // tile of the update kernel
-constexpr int ET = 64;   // tile of the extension kernel
-constexpr int EC = 32;   // candidates per pass
+constexpr int TT = 32;   // tile of the update and compaction kernels
 
-// Persistent grid; one item = 256 vertices i of one walker-spin, all
-// candidates c: clears the reduction targets (the FP64 path's Gc / Xr, and
-// the candidate-block rows of Gc) and tabulates the candidate factors V and U
-// once per window (the tile kernels then read them instead of interpolating;
-// the tensor-core path takes U only in its split form).  The mixed path interpolates on the split grid
-// time (FP32 arithmetic), the FP64 path in FP64.
+// Persistent grid; one item = 32 vertices i of one walker-spin, the candidates
+// dealt out over the eight warps: tabulates the candidate factors V and U once
+// per window (the products then read them instead of interpolating; the
+// tensor-core path takes U only in its split form), and on the mixed path
+// clears the candidate-block rows of Gc, which k_cand_cc adds into.  The mixed
+// path interpolates on the split grid time (FP32 arithmetic), the FP64 path in
+// FP64, where the ~20 FP64 operations of an entry on two FP64 lanes per SM
+// bound the kernel: with 256 vertices an item, one walker of order 310 kept 4
+// SMs busy for 54 us.
+constexpr int CZ = 32;
+
 __global__ void __launch_bounds__(256) k_cand_zero(Config cfg) {
-  __shared__ GridTime s_gc[KS_MAX];
-  __shared__ double s_tc[KS_MAX];
-  __shared__ int s_rc[KS_MAX];
+  __shared__ GridTime s_gc[KS_MAX], s_gi[CZ];
+  __shared__ double s_tc[KS_MAX], s_ti[CZ], s_em1[CZ];
+  __shared__ int s_rc[KS_MAX], s_ri[CZ], s_si[CZ];
   for_each_item(
       2 * cfg.n_walkers,
       [&](int s) -> long long {
         const WalkerDev& w = cfg.W[s >> 1];
         // columns up to n + n_cand (candidate-block targets) and up to the
         // 32-column padding of the tensor-core extension's last K chunk
-        return (w.active && w.n_cand > 0) ? blocks_of(max(w.n + w.n_cand, (w.n + 31) & ~31), 256) : 0;
+        return (w.active && w.n_cand > 0) ? blocks_of(max(w.n + w.n_cand, (w.n + 31) & ~31), CZ) : 0;
       },
       [&](int s, int item) {
         const WalkerDev& w = cfg.W[s >> 1];
         const int sp = s & 1, n = w.n, ld = w.cap, nc_ = w.n_cand, par = w.parity;
         const ProblemDev& pb = cfg.P[w.problem];
         const bool mixed = cfg.prec == PREC_MIXED;
-        __syncthreads();  // the previous item of this block is done with the candidate table
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        const int i = item * CZ + lane;
+        __syncthreads();  // the previous item of this block is done with the shared tables
         for (int c = threadIdx.x; c < nc_; c += 256) {
           s_rc[c] = w.vsite[par][n + c];
           s_tc[c] = w.vtau[par][n + c];
           if (mixed) s_gc[c] = grid_time(s_tc[c], pb.tau_scale);
         }
+        if (warp == 7 && i < n) {
+          const int si = w.vs[par][i];
+          s_si[lane] = si;
+          s_ri[lane] = w.vsite[par][i];
+          s_ti[lane] = w.vtau[par][i];
+          s_em1[lane] = si != 0 ? expV(pb, sp, si) - 1.0 : 0.0;
+          if (mixed) s_gi[lane] = grid_time(s_ti[lane], pb.tau_scale);
+        }
         __syncthreads();
-        const int i = item * 256 + threadIdx.x;
         // split V for the tensor-core extension: [hi | lo] planes x KS_MAX rows x ld columns
         float* Vop = cfg.ext_tc ? reinterpret_cast<float*>(w.Aop[sp]) : nullptr;
         float* Uop = cfg.ext_tc ? reinterpret_cast<float*>(w.Bop[sp]) : nullptr;
         if (i >= n) {
-          if (i < n + nc_)  // targets of the candidate block (k_cand_cc adds into them)
-            for (int c = 0; c < nc_; ++c) w.Gc[sp][(size_t)c * ld + i] = 0.0;
+          if (mixed && i < n + nc_)  // targets of the candidate block
+            for (int c = warp; c < nc_; c += 8) w.Gc[sp][(size_t)c * ld + i] = 0.0;
           if (Vop && i < ((n + 31) & ~31))  // K padding of the last chunk: finite zeros
-            for (int c = 0; c < nc_; ++c) {
+            for (int c = warp; c < nc_; c += 8) {
               Vop[(size_t)c * ld + i] = 0.f;
               Vop[(size_t)(KS_MAX + c) * ld + i] = 0.f;
               Uop[(size_t)c * ld + i] = 0.f;
@@ -203,21 +205,15 @@ __global__ void __launch_bounds__(256) k_cand_zero(Config cfg) {
             }
           return;
         }
-        const int si = w.vs[par][i], ri = w.vsite[par][i];
-        const double ti = w.vtau[par][i];
-        const double em1 = si != 0 ? expV(pb, sp, si) - 1.0 : 0.0;
-        const GridTime gi = grid_time(ti, pb.tau_scale);
-        const float em1f = (float)em1;
-        // unrolled: the table loads of several candidates are in flight together
+        const int si = s_si[lane], ri = s_ri[lane];
+        if (mixed) {
+          const GridTime gi = s_gi[lane];
+          const float em1f = (float)s_em1[lane];
+          // unrolled: the table loads of several candidates are in flight together
 #pragma unroll 4
-        for (int c = 0; c < nc_; ++c) {
-          const size_t o = (size_t)c * ld + i;
-          if (!mixed) {  // targets of the FP64 path's atomics (the mixed-path kernels store rows < n whole)
-            w.Gc[sp][o] = 0.0;
-            w.Xr[sp][o] = 0.0;
-          }
-          const int rc = s_rc[c];
-          if (mixed) {
+          for (int c = warp; c < nc_; c += 8) {
+            const size_t o = (size_t)c * ld + i;
+            const int rc = s_rc[c];
             float v = 0.0f, u = 0.0f;
             if (si != 0) {
               v = g0_interp_grid(g0f_row(pb, sp, __ldg(pb.site_sub + ri * pb.nc + rc)), pb.n_tau, gi, s_gc[c]);
@@ -234,110 +230,22 @@ __global__ void __launch_bounds__(256) k_cand_zero(Config cfg) {
               Uop[(size_t)c * ld + i] = hu;
               Uop[(size_t)(KS_MAX + c) * ld + i] = lu;
             }
-          } else {
+          }
+        } else {
+          const double ti = s_ti[lane], em1 = s_em1[lane];
+#pragma unroll 2
+          for (int c = warp; c < nc_; c += 8) {
+            const int rc = s_rc[c];
             double v = 0.0, u = 0.0;
             if (si != 0) {
               v = g0_pair(pb, sp, ri, ti, rc, s_tc[c]);
               u = g0_pair(pb, sp, rc, s_tc[c], ri, ti) * em1;
             }
-            w.Vb[sp][o] = v;
-            w.Ub[sp][o] = u;
+            w.Vb[sp][(size_t)c * ld + i] = v;
+            w.Ub[sp][(size_t)c * ld + i] = u;
           }
         }
       });
-}
-
-template <typename T, typename A>
-__device__ __forceinline__ void cand_ext_tile(const Config& cfg, int wi, int sp, int tile);
-
-// Persistent grid over (walker-spin, 64 x 64 tile of N).
-template <typename T, typename A>
-__global__ void __launch_bounds__(256) k_cand_ext(Config cfg) {
-  for_each_item(
-      2 * cfg.n_walkers,
-      [&](int s) -> long long {
-        const WalkerDev& w = cfg.W[s >> 1];
-        const long long t = (w.n + ET - 1) / ET;
-        return (w.active && w.n_cand > 0) ? t * t : 0;
-      },
-      [&](int s, int item) { cand_ext_tile<T, A>(cfg, s >> 1, s & 1, item); });
-}
-
-template <typename T, typename A>
-__device__ __forceinline__ void cand_ext_tile(const Config& cfg, int wi, int sp, int tile) {
-  const WalkerDev& w = cfg.W[wi];
-  const int n = w.n, nc_ = w.n_cand;
-  const int tiles = (n + ET - 1) / ET;
-  const int ti = tile / tiles, tj = tile - ti * tiles;
-  const int i0 = ti * ET, j0 = tj * ET;
-  const int ld = w.cap, par = w.parity;
-  const T* __restrict__ N = (const T*)w.N[par][sp];
-  // Shared tiles: N[i][j] and its transpose (so that both products read two
-  // adjacent outputs' operands with one vector load), V[j][c], U^T[i][c].
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  A(*Ns)[ET] = reinterpret_cast<A(*)[ET]>(smem_raw);          // [i][j]
-  A(*Vs)[EC] = reinterpret_cast<A(*)[EC]>(Ns + ET);           // [j][c]
-  A(*Ut)[EC] = Vs + ET;                                       // [i][c]
-  A(*Nt)[ET + 1] = reinterpret_cast<A(*)[ET + 1]>(Ut + ET);   // [j][i], padded: conflict-free transpose
-  const int tid = threadIdx.x;
-  __syncthreads();  // the previous tile of this block is done with the shared tiles
-  for (int e = tid; e < ET * ET; e += 256) {
-    const int r = e / ET, cc = e - r * ET;
-    const int i = i0 + r, j = j0 + cc;
-    const A v = (i < n && j < n) ? ldA<A>(N, (size_t)i * ld + j) : (A)0;
-    Ns[r][cc] = v;
-    Nt[cc][r] = v;
-  }
-  // thread: outputs 2 rows (or columns) x 4 candidates
-  const int tp = tid & 31, tc = tid >> 5;  // pair index, candidate quad (uniform per warp)
-  for (int cb = 0; cb < nc_; cb += EC) {
-    __syncthreads();
-    for (int e = tid; e < ET * EC; e += 256) {
-      const int r = e & (ET - 1), c = e >> 6;  // r fastest: coalesced rows of V and U
-      const int j = j0 + r, i = i0 + r, cg = cb + c;
-      const bool okc = cg < nc_;
-      Vs[r][c] = (okc && j < n) ? reinterpret_cast<const A*>(w.Vb[sp])[(size_t)cg * ld + j] : (A)0;
-      Ut[r][c] = (okc && i < n) ? reinterpret_cast<const A*>(w.Ub[sp])[(size_t)cg * ld + i] : (A)0;
-    }
-    __syncthreads();
-    A g[2][4], x[2][4];
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) g[a][b] = x[a][b] = (A)0;
-    // G partial: rows 2 tp, 2 tp + 1 of the tile, candidates 4 tc .. 4 tc + 3 (sum over j);
-    // X partial: columns 2 tp, 2 tp + 1, same candidates (sum over i).
-#pragma unroll 4
-    for (int k = 0; k < ET; ++k) {
-      const A n0 = Nt[k][2 * tp], n1 = Nt[k][2 * tp + 1];      // N[2tp][k], N[2tp+1][k]
-      const A m0 = Ns[k][2 * tp], m1 = Ns[k][2 * tp + 1];      // N[k][2tp], N[k][2tp+1]
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const A v = Vs[k][4 * tc + b], u = Ut[k][4 * tc + b];
-        g[0][b] += n0 * v;
-        g[1][b] += n1 * v;
-        x[0][b] += u * m0;
-        x[1][b] += u * m1;
-      }
-    }
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int cg = cb + 4 * tc + b;
-      if (cg < nc_) {
-#pragma unroll
-        for (int a = 0; a < 2; ++a) {
-          const int r = 2 * tp + a;
-          if (i0 + r < n) atomicAdd(&w.Gc[sp][(size_t)cg * ld + i0 + r], (double)g[a][b]);
-          if (j0 + r < n) atomicAdd(reinterpret_cast<T*>(w.Xr[sp]) + (size_t)cg * ld + j0 + r, (T)x[a][b]);
-        }
-      }
-    }
-  }
-}
-
-template <typename A>
-constexpr int ext_smem_bytes() {
-  return (int)sizeof(A) * (ET * ET + ET * (ET + 1) + 2 * ET * EC);
 }
 
 // G_ext[n+c', n+c] = X[c',:] . V[c,:] + g0(r_c' - r_c, tau_c' - tau_c)
@@ -348,16 +256,16 @@ constexpr int ext_smem_bytes() {
 // registers while the current one is multiplied.  Thread (tx, ty) of 16 x 16
 // owns c' = ty + 16 a, c = tx + 16 b (a, b < TS / 16).  The segment sums are
 // added into the targets (zeroed by k_cand_zero) with FP64 atomics and
-// segment 0 adds the g0 term.  The products run in the storage type A of N
-// and X.
+// segment 0 adds the g0 term.  Mixed path; the FP64 path has k_cc64.
 constexpr int CC_SEG = 128;
 constexpr int CC_KC = 32;
 
 __device__ __forceinline__ int cc_tile(int nc_) { return nc_ <= 32 ? 32 : 64; }
 
-template <typename A, int TS>
+template <int TS>
 __device__ __forceinline__ void cand_cc_item(const Config& cfg, const WalkerDev& w, int sp, int tile, int seg,
-                                             A (*Xs)[65], A (*Vs)[65]) {
+                                             float (*Xs)[65], float (*Vs)[65]) {
+  using A = float;
   constexpr int MT = TS / 16, PR = TS * CC_KC / 256;  // outputs per thread per axis, loads per thread per operand
   const int n = w.n, nc_ = w.n_cand, ld = w.cap, par = w.parity;
   const int tiles = (nc_ + TS - 1) / TS;
@@ -424,10 +332,9 @@ __device__ __forceinline__ void cand_cc_item(const Config& cfg, const WalkerDev&
   }
 }
 
-template <typename A>
-__global__ void __launch_bounds__(256, sizeof(A) == 4 ? 3 : 2) k_cand_cc(Config cfg) {
-  __shared__ A Xs[CC_KC][65];  // [column][c'], padded: conflict-free transposed stores
-  __shared__ A Vs[CC_KC][65];  // [column][c]
+__global__ void __launch_bounds__(256, 3) k_cand_cc(Config cfg) {
+  __shared__ float Xs[CC_KC][65];  // [column][c'], padded: conflict-free transposed stores
+  __shared__ float Vs[CC_KC][65];  // [column][c]
   for_each_item(
       2 * cfg.n_walkers,
       [&](int s) -> long long {
@@ -440,8 +347,8 @@ __global__ void __launch_bounds__(256, sizeof(A) == 4 ? 3 : 2) k_cand_cc(Config 
         const WalkerDev& w = cfg.W[s >> 1];
         const int segs = (w.n + CC_SEG - 1) / CC_SEG + (w.n == 0);
         const int seg = item % segs, tile = item / segs;
-        if (cc_tile(w.n_cand) == 32) cand_cc_item<A, 32>(cfg, w, s & 1, tile, seg, Xs, Vs);
-        else cand_cc_item<A, 64>(cfg, w, s & 1, tile, seg, Xs, Vs);
+        if (cc_tile(w.n_cand) == 32) cand_cc_item<32>(cfg, w, s & 1, tile, seg, Xs, Vs);
+        else cand_cc_item<64>(cfg, w, s & 1, tile, seg, Xs, Vs);
       });
 }
 
@@ -1478,22 +1385,20 @@ template <typename T, typename A>
 static int launch_group_t(int group, const Config& cfg, int max_cap, cudaStream_t st) {
   const int W = cfg.n_walkers;
   const long long S = 2LL * W;  // walker-spin pairs
-  const long long t64 = (max_cap + ET - 1) / ET, t32 = (max_cap + TT - 1) / TT;
+  const long long t32 = (max_cap + TT - 1) / TT;
   const long long kc = blocks_of((long long)cfg.ks * max_cap, 256);
   switch (group) {
     case GROUP_PROPOSE:
       k_begin<<<W, 128, 0, st>>>(cfg);
       return 1;
     case GROUP_EXTEND:
-      k_cand_zero<<<persist_grid((const void*)k_cand_zero, S * kc, 256), 256, 0, st>>>(cfg);
+      k_cand_zero<<<persist_grid((const void*)k_cand_zero, S * blocks_of(max_cap, CZ), 256), 256, 0, st>>>(cfg);
       if (cfg.prec == PREC_MIXED) {
         int k = launch_ext_mixed(cfg, max_cap, st);
-        k_cand_cc<A><<<persist_grid((const void*)k_cand_cc<A>, S * 16, 256), 256, 0, st>>>(cfg);
+        k_cand_cc<<<persist_grid((const void*)k_cand_cc, S * 16, 256), 256, 0, st>>>(cfg);
         return 2 + k;
       }
-      k_cand_ext<T, A><<<grid_for(S * t64 * t64), 256, ext_smem_bytes<A>(), st>>>(cfg);
-      k_cand_cc<A><<<grid_for(S * 16), 256, 0, st>>>(cfg);
-      return 3;
+      return 1 + launch_ext64(cfg, max_cap, st);
     case GROUP_METROPOLIS: {
       if (sizeof(T) == 8 || cfg.gamma_fp64) {
         launch_metropolis64(cfg, st);
@@ -1530,13 +1435,8 @@ static int launch_group_t(int group, const Config& cfg, int max_cap, cudaStream_
 }
 
 cudaError_t setup_window_kernels() {
-  cudaError_t e = cudaFuncSetAttribute(k_cand_ext<double, double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       ext_smem_bytes<double>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_cand_ext<float, float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             ext_smem_bytes<float>());
   const int msm = (int)sizeof(double) * 2 * METRO_SMEM_KS * (METRO_SMEM_KS | 1);
-  if (e == cudaSuccess) e = setup_metropolis64();
+  cudaError_t e = setup_metropolis64();
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_metropolis<float, float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, msm);
   return e;

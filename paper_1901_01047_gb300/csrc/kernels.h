@@ -11,7 +11,7 @@ namespace dca {
 // Kernel groups of one window (and the per-window extras), timed separately.
 enum Group : int {
   GROUP_PROPOSE = 0,         // k_begin
-  GROUP_EXTEND = 1,          // k_cand_zero, k_cand_ext (mixed: k_ext_g, k_ext_x), k_cand_cc
+  GROUP_EXTEND = 1,          // k_cand_zero, k_ext64, k_cc64 (mixed: k_ext_g, k_ext_x, k_cand_cc)
   GROUP_METROPOLIS = 2,      // k_metropolis
   GROUP_UPDATE = 3,          // the rank-l update of N
   GROUP_MEASURE = 4,         // k_meas_*
@@ -82,6 +82,7 @@ int sm_grid(long long items, int per_sm);
 // cached per kernel), at most `items`.
 int persist_grid(const void* fn, long long items, int block, size_t smem = 0);
 // Candidate extension of the mixed path: the two streaming passes over N.
+int launch_ext64(const Config& cfg, int max_cap, cudaStream_t st);  // FP64 path: both passes and the candidate block
 int launch_ext_mixed(const Config& cfg, int max_cap, cudaStream_t st);
 // Tensor-core N update (mixed precision): kernel attributes, tile width for
 // a submatrix size, tensor maps of one walker ([spin][A, B, N0, N1]), the
