@@ -36,6 +36,7 @@
 // come from one 64-bit integer product, and the phase (2n + 1) tau / beta
 // modulo 2 from another, so the sample loops of both variants run without
 // FP64 arithmetic (FP64 is 1/64 of the FP32 rate on this GPU).
+#include <algorithm>
 #include <cstdint>
 #include <type_traits>
 
@@ -235,6 +236,117 @@ __global__ void __launch_bounds__(256) k_meas_nfft(Config cfg) {
       });
 }
 
+// The spreading of the FP64 path with a private grid per warp and no atomics:
+// k_meas_nfft spends its time in the compare-and-swap loops that FP64
+// additions to shared memory are, 24 a sample.  A warp prepares 32 samples of a
+// row of N, one a lane (the weights by the recurrence of spread_sample), hands
+// the weights over through shared memory and adds the samples to its grid one
+// at a time, 24 lanes a sample, with plain loads and stores.  At the end of an
+// item (rb rows, dealt out over the warps) the grids are summed into the
+// walker's and cleared.  What is left is the FP64 work of the weights and the
+// load-add-store latency of a sample: 48 walkers of 4 sites, order 41, 64
+// frequencies, 240 -> 113 us a measurement.  (In FP32 the additions to shared memory
+// are cheap and the same layout was 2.5 times slower than k_meas_nfft.)
+constexpr int SPREAD_WARPS = 8;
+constexpr int SPREAD_WST = 33;  // odd stride of the weight rows
+constexpr size_t SPREAD_WEIGHT_BYTES = sizeof(double) * 2 * NFFT_MSP_MAX * SPREAD_WST;
+
+__global__ void __launch_bounds__(32 * SPREAD_WARPS) k_nfft_spread64(Config cfg, int rb, int stride) {
+  extern __shared__ __align__(16) unsigned char nfft_raw[];
+  __shared__ double s_e3[NFFT_MSP_MAX + 1];
+  const int L = cfg.nfft_L, msp = cfg.nfft_msp;
+  const double a = 0.75 * 3.14159265358979323846 / (double)msp;  // pi (R - 1/2) / (R M_sp), R = 2
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  double* const grids = reinterpret_cast<double*>(nfft_raw);
+  double* const g = grids + (size_t)warp * stride;
+  double* const wts = grids + (size_t)nwarps * stride + (size_t)warp * (2 * NFFT_MSP_MAX * SPREAD_WST);
+  if (threadIdx.x <= msp) s_e3[threadIdx.x] = exp(-a * threadIdx.x * threadIdx.x);
+  for (int e = threadIdx.x; e < nwarps * stride; e += blockDim.x) grids[e] = 0.0;
+  __syncthreads();
+  for_each_item(
+      2 * cfg.n_walkers,
+      [&](int s) -> long long {
+        const WalkerDev& w = cfg.W[s >> 1];
+        return wants_nfft(cfg, w) ? blocks_of(w.n, rb) : 0;
+      },
+      [&](int s, int item) {
+        const WalkerDev& w = cfg.W[s >> 1];
+        const int sp = s & 1, n = w.n, ld = w.cap, par = w.parity;
+        const ProblemDev& pb = cfg.P[w.problem];
+        const int nc = pb.nc;
+        const double* N = (const double*)w.N[par][sp];
+        const unsigned long long* vx = w.vx;
+        const double scale = w.sign / (pb.beta * (double)nc);
+        const int i1 = min(n, (item + 1) * rb);
+        for (int i = item * rb + warp; i < i1; i += nwarps) {
+          const unsigned long long wi = vx[i];
+          if (wi == 0ull) continue;  // dead row: its factor e^{V} - 1 is zero
+          const double fi = (expV(pb, sp, w.vs[par][i]) - 1.0) * scale;
+          const unsigned long long Xi = wi >> 8;
+          const int* sub_row = pb.site_sub + (int)((wi & 0xffull) - 1ull) * nc;
+          const double* Nrow = N + (size_t)i * ld;
+          for (int j0 = 0; j0 < n; j0 += 32) {
+            // this lane's sample: value m at grid position l0 + d of the row at `base`
+            const int j = j0 + lane;
+            const unsigned long long wj = j < n ? __ldg(vx + j) : 0ull;
+            const bool live = wj != 0ull;  // else a dead column: the unit vector, zero after the factor
+            int base = 0, l0 = 0;
+            if (live) {
+              const unsigned long long Xj = wj >> 8;
+              // t = tau_i - tau_j, moved into [0, beta) with the antiperiodic sign
+              double m = fi * Nrow[j];
+              if (Xi < Xj) m = -m;
+              const unsigned long long sh = ((Xi - Xj) & X56_MASK) << 8;  // frac(t / beta) in 2^-64 units
+              l0 = (int)__umul64hi(sh, (unsigned long long)L);
+              const double d = frac64<double>(sh * (unsigned long long)L);
+              base = __ldg(sub_row + (int)((wj & 0xffull) - 1ull)) * L;
+              // weights e1 e2^k e3[|k|] of the points l0 + k, k = -msp .. msp - 1
+              const double e1 = m * exp(-a * d * d), e2 = exp(2.0 * a * d), e2i = 1.0 / e2;
+              double p = e1, q = e1 * e2;
+#pragma unroll 4
+              for (int k = 0; k < msp; ++k) {
+                wts[(msp - k) * SPREAD_WST + lane] = p * s_e3[k];
+                p *= e2i;
+                if (k + 1 < msp) wts[(msp + k + 1) * SPREAD_WST + lane] = q * s_e3[k + 1];
+                q *= e2;
+              }
+              wts[lane] = p * s_e3[msp];
+            }
+            __syncwarp();
+            const unsigned mask = __ballot_sync(0xffffffffu, live);
+            const int cnt = min(32, n - j0);
+            for (int q = 0; q < cnt; ++q) {
+              const int bq = __shfl_sync(0xffffffffu, base, q), lq = __shfl_sync(0xffffffffu, l0, q);
+              if (((mask >> q) & 1u) && lane < 2 * msp) {
+                double v = wts[lane * SPREAD_WST + q];
+                int l = lq + lane - msp;
+                if (l < 0) {
+                  l += L;
+                  v = -v;
+                } else if (l >= L) {
+                  l -= L;
+                  v = -v;
+                }
+                g[bq + l] += v;
+              }
+              __syncwarp();
+            }
+          }
+        }
+        __syncthreads();
+        double* gglob = w.Mgrid + (size_t)sp * nc * L;
+        for (int e = threadIdx.x; e < nc * L; e += blockDim.x) {
+          double v = 0.0;
+          for (int h = 0; h < nwarps; ++h) {
+            v += grids[(size_t)h * stride + e];
+            grids[(size_t)h * stride + e] = 0.0;
+          }
+          if (v != 0.0) atomicAdd(gglob + e, v);
+        }
+        __syncthreads();  // the grids are clear before the next item
+      });
+}
+
 // Read-out: M(dr, i w_n) = [sum_l g_l e^{i w_n l h}] / phi_hat(w_n h) for every
 // walker, spin, difference and frequency; out [w][2][nc][n_omega][re, im]
 // at offset base[w].  The phases are exact multiples of pi / L ((2n + 1) l
@@ -339,6 +451,7 @@ __global__ void __launch_bounds__(256) k_nfft_finish_direct(Config cfg, const lo
 // Largest grid staged in shared memory per block (bytes); larger grids are
 // accumulated in global memory directly.
 constexpr size_t NFFT_SMEM_MAX = 160 * 1024;
+constexpr size_t NFFT_SPREAD_SMEM_MAX = 220 * 1024;  // grids and weights of the FP64 spreading
 constexpr size_t NFFT_FINISH_SMEM_MAX = 200 * 1024;  // tables of the read-out transform
 
 size_t nfft_smem_bytes(const Config& cfg, int max_nc) {
@@ -358,6 +471,8 @@ cudaError_t setup_nfft() {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_meas_nfft<float, float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)NFFT_SMEM_MAX);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_nfft_spread64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)NFFT_SPREAD_SMEM_MAX);
   return e;
 }
 
@@ -368,6 +483,18 @@ int launch_meas_nfft(const Config& cfg, int max_cap, int max_nc, cudaStream_t st
   if (cfg.freq_dft) return 1 + launch_meas_ndft(cfg, max_cap, max_nc, st);
   const long long items = 2LL * cfg.n_walkers * blocks_of(max_cap, NFFT_RB);
   const size_t smem = nfft_smem_bytes(cfg, max_nc);
+  // FP64: a grid per warp where at least two fit an SM's shared memory; larger
+  // grids (n_omega in the hundreds with 16 sites) are staged once per block or
+  // not at all.  Two rows a warp and item: the sum over the grids at its end
+  // costs about a fifth of a row.
+  const size_t per_warp = smem + SPREAD_WEIGHT_BYTES;
+  const int nw = (int)std::min<size_t>(SPREAD_WARPS, NFFT_SPREAD_SMEM_MAX / per_warp);
+  if (cfg.prec != PREC_MIXED && nw >= 2) {
+    const int per_sm = std::max(1, (int)(NFFT_SPREAD_SMEM_MAX / (nw * per_warp))), rb = 2 * nw;
+    const int grid = sm_grid(2LL * cfg.n_walkers * blocks_of(max_cap, rb), per_sm);
+    k_nfft_spread64<<<grid, 32 * nw, nw * per_warp, st>>>(cfg, rb, max_nc * cfg.nfft_L);
+    return 2;
+  }
   if (smem <= NFFT_SMEM_MAX) {
     if (cfg.prec == PREC_MIXED) {
       const void* fn = (const void*)k_meas_nfft<float, float, true>;
