@@ -309,223 +309,6 @@ __global__ void __launch_bounds__(256) k_meas_b(Config cfg) {
       });
 }
 
-// Correction term as a product: rows (x, tau_a), inner index the vertex i,
-// columns the reference site r':
-//   C[(x, a), r'] = sum_i g0(x - r_i, tau_a - tau_i) b_i(r'),
-// scattered to Gtmp[sp][x - r'][a] (FP64 atomics).  The g0 factor is
-// interpolated on the fly (FP64 path: FP64; mixed path: FP32 on the split
-// grid time, with the tau_a and tau_i grid times formed once per tile).  A is
-// the arithmetic type of the products, MR >= nc the reference-site tile.
-// Item = (site x, block of MT tau points) of one walker-spin, block 256.
-constexpr int MT = 64;   // tau points per item
-constexpr int MK = 32;   // vertices per step
-
-template <typename A, int MR>
-__device__ __forceinline__ void meas_gemm_item(const Config& cfg, int wi, int sp, int item);
-
-// One kernel per reference-site tile MR, each taking the walkers whose
-// cluster falls in its class (MR / 2 < nc <= MR; nc <= 16 for MR = 16): the
-// register allocation of each follows its own tile.
-template <typename A, int MR>
-__global__ void __launch_bounds__(256) k_meas_gemm(Config cfg) {
-  for_each_item(
-      2 * cfg.n_walkers,
-      [&](int s) -> long long {
-        const WalkerDev& w = cfg.W[s >> 1];
-        const int nc = cfg.P[w.problem].nc;
-        const bool mine = MR == 16 ? nc <= 16 : (nc > MR / 2 && nc <= MR);
-        return (wants_measure(w) && mine) ? (long long)nc * blocks_of(cfg.n_tau_meas, MT) : 0;
-      },
-      [&](int s, int item) { meas_gemm_item<A, MR>(cfg, s >> 1, s & 1, item); });
-}
-
-// Item = (reference site x, MT tau points): the tiles of MK vertices pass
-// through shared memory.  On the FP32 path in two stages: while the tile t
-// is multiplied, the table values of tile t + 1 are filled in and the vertex
-// records of tile t + 2 prepared, one barrier per tile; the FP64 path keeps
-// one stage (its tiles would not fit twice in static shared memory).
-template <typename A, int MR>
-__device__ __forceinline__ void meas_gemm_item(const Config& cfg, int wi, int sp, int item) {
-  constexpr bool kGrid = sizeof(A) == 4;
-  constexpr int NS = kGrid ? 2 : 1;  // stages
-  const WalkerDev& w = cfg.W[wi];
-  const ProblemDev& pb = cfg.P[w.problem];
-  const int nc = pb.nc, ntm = cfg.n_tau_meas, n = w.n, par = w.parity, ld = w.cap;
-  const int tblocks = (ntm + MT - 1) / MT;
-  const int x = item / tblocks, a0 = (item - x * tblocks) * MT;
-  __shared__ A As[NS][MT][MK + 1];
-  __shared__ __align__(16) A Bs[NS][MK][MR];  // rows of MR values: a thread's MR / 4 sites are contiguous
-  __shared__ GridTime s_ga[MT], s_gi[NS][MK];
-  __shared__ int s_row[NS][MK];               // table row of g0(x - r_i, .), -1 for a dead vertex
-  __shared__ int s_ph[NS][MK], s_mb[NS][MK];  // phase-table path: phase p_i and m offset of vertex i
-  __shared__ float s_fw[NS][MK];              // and its interpolation weight
-  const int q = kGrid ? pb.meas_q : 0;
-  const int tid = threadIdx.x;
-  const int ta = tid & (MT - 1), tr = tid >> 6;  // 4 groups of reference sites
-  // products summed in A within a tile of MK vertices; the tile sums in FP64
-  // (FP64 path) or in double-float (FP32 path: an error-free FP32 two-sum per
-  // tile instead of a conversion and an add on GB300's scarce FP64 units)
-  double tot[MR / 4];
-  float th[MR / 4], tl[MR / 4];
-#pragma unroll
-  for (int m = 0; m < MR / 4; ++m) {
-    tot[m] = 0.0;
-    th[m] = tl[m] = 0.0f;
-  }
-  const int* vsite = w.vsite[par];
-  const double* vtau = w.vtau[par];
-  const int* vs = w.vs[par];
-  const int np1 = pb.n_tau + 1;
-  const double* row_base = pb.g0 + (size_t)sp * nc * np1;
-
-  // vertex records of the tile at i0 into stage b (threads tid < MK)
-  auto prep = [&](int i0, int b) {
-    if (tid < MK) {
-      const int i = i0 + tid;
-      const bool live = i < n && vs[i] != 0;
-      s_row[b][tid] = live ? __ldg(pb.site_sub + x * nc + vsite[i]) : -1;
-      if (kGrid && live) {
-        const GridTime gi = grid_time(vtau[i], pb.tau_scale);
-        s_gi[b][tid] = gi;
-        if (q > 0) {
-          // grid offset of tau_a - tau_i: l = q a + c, c = q/2 - gi.i - (gi.f > 0), weight 1 - gi.f
-          const int c = q / 2 - gi.i - (gi.f > 0.0f ? 1 : 0);
-          const int p = ((c % q) + q) % q;
-          s_ph[b][tid] = p;
-          s_mb[b][tid] = (c - p) / q;
-          s_fw[b][tid] = gi.f > 0.0f ? 1.0f - gi.f : 0.0f;
-        }
-      }
-    }
-  };
-  // table values g0(x - r_i, tau_a - tau_i) and the rows b_i of the tile at i0 into stage b
-  auto fill = [&](int i0, int b) {
-    if (q > 0) {
-      // phase table: consecutive threads take consecutive tau points of one
-      // vertex, i.e. consecutive entries of one phase row
-      const size_t mrow = (size_t)ntm + 1;
-      const float* gm = pb.g0m + (size_t)sp * q * nc * mrow;
-      for (int e = tid; e < MT * MK; e += 256) {
-        const int il = e / MT, al = e - il * MT;
-        const int a = a0 + al, d = s_row[b][il];
-        A v = (A)0;
-        if (a < ntm && d >= 0) {
-          const int p = s_ph[b][il];
-          int m = a + s_mb[b][il];
-          float sgn = 1.0f;
-          if (m < 0) {  // tau_a - tau_i < 0: antiperiodic continuation
-            m += ntm;
-            sgn = -1.0f;
-          }
-          const float lo = __ldg(gm + ((size_t)p * nc + d) * mrow + m);
-          const float hi = p + 1 < q ? __ldg(gm + ((size_t)(p + 1) * nc + d) * mrow + m)
-                                     : __ldg(gm + (size_t)d * mrow + m + 1);
-          v = (A)(sgn * (lo + s_fw[b][il] * (hi - lo)));
-        }
-        As[b][al][il] = v;
-      }
-    } else {
-      for (int e = tid; e < MT * MK; e += 256) {
-        const int al = e / MK, il = e - al * MK;
-        const int a = a0 + al, d = s_row[b][il];
-        A v = (A)0;
-        if (a < ntm && d >= 0) {
-          const double* row = row_base + (size_t)d * np1;
-          if (kGrid) {
-            v = (A)g0_interp_grid(g0f_row(pb, sp, d), pb.n_tau, s_ga[al], s_gi[b][il]);
-          } else {
-            const double ta_ = ((double)a + 0.5) * pb.beta / (double)ntm;
-            v = (A)g0_interp(row, pb.n_tau, pb.beta, pb.tau_scale, ta_ - vtau[i0 + il]);
-          }
-        }
-        As[b][al][il] = v;
-      }
-    }
-    for (int e = tid; e < MK * MR; e += 256) {
-      const int il = e / MR, rp = e - il * MR;
-      const int i = i0 + il;
-      Bs[b][il][rp] = (i < n && rp < nc) ? reinterpret_cast<const A*>(w.bvec)[((size_t)sp * nc + rp) * ld + i] : (A)0;
-    }
-  };
-  // products of stage b, added to the tile sums
-  auto compute = [&](int b) {
-    A acc[MR / 4];
-#pragma unroll
-    for (int m = 0; m < MR / 4; ++m) acc[m] = (A)0;
-#pragma unroll 4
-    for (int k = 0; k < MK; ++k) {
-      const A g = As[b][ta][k];
-      // sites MR/4 tr .. MR/4 tr + MR/4 - 1: the same row segment for the whole
-      // warp (a broadcast), read as 16-byte vectors on the FP32 path
-      if constexpr (sizeof(A) == 4) {
-#pragma unroll
-        for (int m4 = 0; m4 < MR / 16; ++m4) {
-          const float4 bv = *reinterpret_cast<const float4*>(&Bs[b][k][tr * (MR / 4) + 4 * m4]);
-          acc[4 * m4] += g * bv.x;
-          acc[4 * m4 + 1] += g * bv.y;
-          acc[4 * m4 + 2] += g * bv.z;
-          acc[4 * m4 + 3] += g * bv.w;
-        }
-      } else {
-#pragma unroll
-        for (int m = 0; m < MR / 4; ++m) acc[m] += g * Bs[b][k][tr * (MR / 4) + m];
-      }
-    }
-    if constexpr (sizeof(A) == 4) {
-#pragma unroll
-      for (int m = 0; m < MR / 4; ++m) {
-        const float s1 = __fadd_rn(th[m], (float)acc[m]);
-        const float bb = __fsub_rn(s1, th[m]);
-        tl[m] += __fadd_rn(__fsub_rn(th[m], __fsub_rn(s1, bb)), __fsub_rn((float)acc[m], bb));
-        th[m] = s1;
-      }
-    } else {
-#pragma unroll
-      for (int m = 0; m < MR / 4; ++m) tot[m] += (double)acc[m];
-    }
-  };
-
-  __syncthreads();  // the previous item of this block is done with the shared tiles
-  if (kGrid && tid < MT) s_ga[tid] = grid_time(((double)(a0 + tid) + 0.5) * pb.beta / (double)ntm, pb.tau_scale);
-  if constexpr (NS == 2) {
-    if (n > 0) {
-      prep(0, 0);
-      if (MK < n) prep(MK, 1);
-      __syncthreads();
-      fill(0, 0);
-      __syncthreads();
-      for (int i0 = 0, t = 0; i0 < n; i0 += MK, ++t) {
-        const int b = t & 1;
-        if (i0 + MK < n) fill(i0 + MK, b ^ 1);     // reads the records of stage b ^ 1
-        compute(b);
-        if (i0 + 2 * MK < n) prep(i0 + 2 * MK, b);  // stage b's records were read one tile ago
-        __syncthreads();
-      }
-    }
-  } else {
-    for (int i0 = 0; i0 < n; i0 += MK) {
-      __syncthreads();
-      prep(i0, 0);
-      __syncthreads();
-      fill(i0, 0);
-      __syncthreads();
-      compute(0);
-    }
-  }
-  const int a = a0 + ta;
-  if (a < ntm) {
-#pragma unroll
-    for (int m = 0; m < MR / 4; ++m) {
-      const int rp = tr * (MR / 4) + m;
-      if (rp < nc) {
-        const int d = __ldg(pb.site_sub + x * nc + rp);
-        const double v = sizeof(A) == 4 ? (double)th[m] + (double)tl[m] : tot[m];
-        atomicAdd(&w.Gtmp[((size_t)sp * nc + d) * ntm + a], v);
-      }
-    }
-  }
-}
-
 // Gacc[sp][dr][a] += sign * (-G), G = g0(dr, tau_a) + Gtmp / Nc; Gtmp cleared.
 // grid = (blocks, walkers), thread per (sp, dr, a).
 __global__ void __launch_bounds__(256) k_meas_acc(Config cfg) {
@@ -819,22 +602,11 @@ int launch_measure(const Config& cfg, int max_cap, int max_nc, cudaStream_t st) 
     k_meas_b<float, float><<<persist_grid((const void*)k_meas_b<float, float>, ib, 256), 256, 0, st>>>(cfg);
   else
     k_meas_b<double, double><<<persist_grid((const void*)k_meas_b<double, double>, ib, 256), 256, 0, st>>>(cfg);
-  const long long ig = S * max_nc * blocks_of(cfg.n_tau_meas, MT);
-#define DCA_MEAS_GEMM(A, MR) k_meas_gemm<A, MR><<<persist_grid((const void*)k_meas_gemm<A, MR>, ig, 256), 256, 0, st>>>(cfg)
-  if (cfg.prec == PREC_MIXED) {
-    DCA_MEAS_GEMM(float, 16);
-    if (max_nc > 16) DCA_MEAS_GEMM(float, 32);
-    if (max_nc > 32) DCA_MEAS_GEMM(float, 64);
-  } else {
-    DCA_MEAS_GEMM(double, 16);
-    if (max_nc > 16) DCA_MEAS_GEMM(double, 32);
-    if (max_nc > 32) DCA_MEAS_GEMM(double, 64);
-  }
-#undef DCA_MEAS_GEMM
+  const int ng = launch_meas_gemm(cfg, max_nc, st);
   k_meas_acc<<<grid_for((long long)W * blocks_of(2LL * max_nc * cfg.n_tau_meas, 256)), 256, 0, st>>>(cfg);
   const int nf = launch_meas_nfft(cfg, max_cap, max_nc, st) + launch_meas_g4(cfg, max_cap, max_nc, st);
   k_meas_finish<<<(W + 127) / 128, 128, 0, st>>>(cfg);
-  return 5 + (max_nc > 16) + (max_nc > 32) + nf;
+  return 4 + ng + nf;
 }
 
 // Read-out of the tau-grid measurement: every walker's accumulator Gacc

@@ -288,7 +288,9 @@ extern "C" DCA_API int dca_walker_create(const dca_walker_params* prm, void* cud
     d.g0 = (const double*)dg;
     d.g0f = (const float*)dgf;
     const int q = (p.n_tau_meas > 0 && d.n_tau % p.n_tau_meas == 0) ? d.n_tau / p.n_tau_meas : 0;
-    if (h->precision == DCA_PREC_MIXED && q >= 2 && q % 2 == 0) {
+    // (row offsets of the phase table are 32-bit)
+    if (h->precision == DCA_PREC_MIXED && q >= 2 && q % 2 == 0 &&
+        (long long)q * pr.nc * (p.n_tau_meas + 1LL) < (1LL << 31)) {
       void* dgm = h->dalloc(sizeof(float) * 2 * (size_t)q * pr.nc * (p.n_tau_meas + 1));
       if (!dgm) {
         h->err = "device allocation of the measurement phase table";
@@ -540,7 +542,8 @@ extern "C" DCA_API int dca_walker_create(const dca_walker_params* prm, void* cud
   h->cfg.m4 = p.n_w4 > 0 ? p.w4_transfer : 0;
   h->q4 = p.n_w4 > 0 ? p.q4_transfer : 0;
 
-  if (dca::setup_window_kernels() != cudaSuccess || dca::setup_nfft() != cudaSuccess) {
+  if (dca::setup_window_kernels() != cudaSuccess || dca::setup_nfft() != cudaSuccess ||
+      dca::setup_meas_gemm() != cudaSuccess) {
     h->err = "kernel attribute setup failed";
     return bail(DCA_ERR_CUDA);
   }
