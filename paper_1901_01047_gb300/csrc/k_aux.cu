@@ -50,38 +50,97 @@ __device__ __forceinline__ double* work_matrix(const Config& cfg, const WalkerDe
   return (double*)w.N[mode == 1 ? w.parity ^ 1 : w.parity][sp];
 }
 
-// Persistent grid; one item = 256 entries of one walker-spin's A.
+// Imaginary times on the g0 grid as fixed-point words X = tau n_tau / beta 2^F,
+// F = 61 - floor(log2(n_tau + 1)), with the rounding error of the FP64 product
+// (an FMA) carried along: a difference of two is exact, its integer part is the
+// table index and its fraction the weight, so that an entry of A costs five
+// FP64 operations and one conversion (weight, table difference, interpolation,
+// factor, split) where the interpolation from the times took about sixteen.
+// 256 walkers of orders 90 to 900: 1.62 -> 1.04 ms a recompute, now bound by the
+// two table gathers of an entry.
+__device__ __forceinline__ int fixed_bits(int n_tau) { return 30 + __clz(n_tau + 1); }
+
+__device__ __forceinline__ long long fixed_time(double tau, double tau_scale, int F) {
+  const double two_f = __longlong_as_double((long long)(1023 + F) << 52);  // 2^F: the products with it are exact
+  const double x = tau * tau_scale, e = fma(tau, tau_scale, -x);
+  return (long long)(x * two_f) + __double2ll_rn(e * two_f);
+}
+
+// FP64 -> unevaluated FP32 pair hi + lo, hi rounded to nearest (about 49 bits).
+// Normal values split by their bits: the FP64 units see one subtraction and
+// one conversion.
+__device__ __forceinline__ float2 split_pair(double a) {
+  const long long u = __double_as_longlong(a) + (1ll << 28);  // round the upper 24 bits, half away from zero
+  const int e = (int)((u >> 52) & 0x7ff) - (1023 - 127);
+  if (e <= 0 || e >= 255) {  // zero, or outside FP32's normal range
+    const float hi = (float)a;
+    return make_float2(hi, (float)(a - (double)hi));
+  }
+  const double hd = __longlong_as_double(u & ~((1ll << 29) - 1));
+  const unsigned f = (unsigned)((u >> 32) & 0x80000000u) | ((unsigned)e << 23) | ((unsigned)(u >> 29) & 0x7fffffu);
+  return make_float2(__uint_as_float(f), (float)(a - hd));
+}
+
+constexpr int BA_R = 32, BA_C = 64;  // rows and columns of a k_build_A item
+
+// Persistent grid; one item = BA_R x BA_C entries of one walker-spin's A, a
+// thread eight rows of a column.  Bound by the FP64 units (two lanes per SM).
 __global__ void __launch_bounds__(256) k_build_A(Config cfg, int mode) {
+  __shared__ long long s_X[BA_R];
+  __shared__ int s_site[BA_R];
   if (blockIdx.x == 0 && threadIdx.x == 0) *cfg.gj_next = 0;  // work queue of the inverse that follows
   for_each_item(
       2 * cfg.n_walkers,
       [&](int s) -> long long {
         const WalkerDev& w = cfg.W[s >> 1];
-        return wants_build(w, mode) ? blocks_of((long long)w.n * w.n, 256) : 0;
+        return wants_build(w, mode) ? blocks_of(w.n, BA_R) * blocks_of(w.n, BA_C) : 0;
       },
       [&](int s, int item) {
-  const WalkerDev& w = cfg.W[s >> 1];
-  const int sp = s & 1;
-  const int n = w.n, ld = w.cap, par = w.parity;
-  const ProblemDev& pb = cfg.P[w.problem];
-  double* A = work_matrix(cfg, w, mode, sp);
-  const int* vsite = w.vsite[par];
-  const double* vtau = w.vtau[par];
-  const int* vs = w.vs[par];
-  const long long idx = (long long)item * 256 + threadIdx.x;
-  if (idx < (long long)n * n) {
-    const int i = (int)(idx / n), j = (int)(idx - (long long)i * n);
-    const double ej = expV(pb, sp, vs[j]);
-    const double g = (i == j) ? g0_diag(pb, sp, vsite[i]) : g0_pair(pb, sp, vsite[i], vtau[i], vsite[j], vtau[j]);
-    const double a = (i == j ? ej : 0.0) - g * (ej - 1.0);
-    if (mode == 1 && cfg.prec == PREC_MIXED && !cfg.recompute_gj) {
-      // Newton recompute: A as an unevaluated FP32 pair hi + lo (~48 bits)
-      const float hi = (float)a;
-      reinterpret_cast<float2*>(A)[(size_t)i * ld + j] = make_float2(hi, (float)(a - (double)hi));
-    } else {
-      A[(size_t)i * ld + j] = a;
-    }
-  }
+        const WalkerDev& w = cfg.W[s >> 1];
+        const int sp = s & 1, n = w.n, ld = w.cap, par = w.parity;
+        const ProblemDev& pb = cfg.P[w.problem];
+        const int nc = pb.nc, n_tau = pb.n_tau, F = fixed_bits(n_tau);
+        const int cblocks = (n + BA_C - 1) / BA_C;
+        const int i0 = (item / cblocks) * BA_R, j = (item % cblocks) * BA_C + (threadIdx.x & (BA_C - 1));
+        double* A = work_matrix(cfg, w, mode, sp);
+        const bool pairs = mode == 1 && cfg.prec == PREC_MIXED && !cfg.recompute_gj;
+        __syncthreads();  // the previous item of this block is done with the row records
+        if (threadIdx.x < BA_R && i0 + threadIdx.x < n) {
+          s_X[threadIdx.x] = fixed_time(w.vtau[par][i0 + threadIdx.x], pb.tau_scale, F);
+          s_site[threadIdx.x] = w.vsite[par][i0 + threadIdx.x];
+        }
+        __syncthreads();
+        if (j >= n) return;
+        const long long Xj = fixed_time(w.vtau[par][j], pb.tau_scale, F), span = (long long)n_tau << F;
+        const int sj = w.vsite[par][j];
+        const double ej = expV(pb, sp, w.vs[par][j]), mej1 = 1.0 - ej;
+        const double* g0 = pb.g0 + (size_t)sp * nc * (size_t)(n_tau + 1);
+        const int rl = threadIdx.x / BA_C;
+#pragma unroll 4
+        for (int u = 0; u < BA_R * BA_C / 256; ++u) {
+          const int r = rl + (256 / BA_C) * u, i = i0 + r;
+          if (i >= n) break;
+          const double* row = g0 + (size_t)__ldg(pb.site_sub + s_site[r] * nc + sj) * (size_t)(n_tau + 1);
+          // g0(tau_i - tau_j): linear interpolation, g0(t - beta) = -g0(t), equal times read as 0+
+          long long D = s_X[r] - Xj;
+          double m = mej1;
+          if (D < 0) {
+            D += span;
+            m = __longlong_as_double(__double_as_longlong(m) ^ (1ll << 63));
+          }
+          int k = (int)(D >> F);
+          const unsigned long long frac = (unsigned long long)D << (64 - F);  // the fraction in 2^-64
+          double f = __longlong_as_double(0x3ff0000000000000ll | (long long)(frac >> 12)) - 1.0;
+          if (k >= n_tau) {
+            k = n_tau - 1;
+            f = 1.0;
+          }
+          const double lo = __ldg(row + k), hi = __ldg(row + k + 1);
+          double a = m * fma(f, hi - lo, lo);
+          if (i == j) a = fma(mej1, g0_diag(pb, sp, sj), ej);
+          if (pairs) reinterpret_cast<float2*>(A)[(size_t)i * ld + j] = split_pair(a);
+          else A[(size_t)i * ld + j] = a;
+        }
       });
 }
 
