@@ -12,7 +12,7 @@
 // issue ~2 FMA per clock per SM against 128 FP32 operations.
 //
 // Buffers (the recompute follows a compaction, all n rows live):
-//   A   Ascr[sp] (FP32 pairs)    -> R  into N[parity ^ 1][sp] (FP32)
+//   A   Ascr[sp] (FP32 pairs)    -> R  into N[parity ^ 1][sp] (FP32; from the digit planes R^T, see k_refine_tc.cu)
 //   N0  N[parity][sp]            -> N1 into Ascr[sp] viewed as FP32
 // k_refine_adopt then measures the drift max|N1 - N0| / max|N1| and copies
 // N1 into N[parity ^ 1][sp] for the parity switch.

@@ -477,19 +477,31 @@ __global__ void __launch_bounds__(192, 1) k_refine_oz(Config cfg) {
         }
       }
       if (stop) break;
-      // R[i, j] = delta_ij - 2^(ea_i + eb_j - 18) (h + l), FP32
+      // R[i, j] = delta_ij - 2^(ea_i + eb_j - 18) (h + l), stored transposed as
+      // two TF32 planes: K-major operands of the correction N0 R (k_correct_tc),
+      // with zeros up to the 32-column padding of its last K step
       const int j = j0 + r;
       if (j < n) {
-        const int eb = w.OzE[sp][ld + j];
-        float* R = (float*)w.N[w.parity ^ 1][sp];
+        const int eb = w.OzE[sp][ld + j], n32 = (n + 31) & ~31;
+        float* Rh = (float*)w.N[w.parity ^ 1][sp] + (size_t)j * ld;
+        float* Rl = reinterpret_cast<float*>(w.Ascr[sp]) + (size_t)ld * ld + (size_t)j * ld;
 #pragma unroll
-        for (int x = 0; x < OZ_BN; ++x) {
-          const int i = i0 + x;
-          if (i < n) {
-            const int e = w.OzE[sp][i] + eb - 2 * OZ_BETA;
-            const float d = __fsub_rn(i == j ? 1.0f : 0.0f, ldexpf(h[x], e));
-            R[(size_t)i * ld + j] = __fsub_rn(d, ldexpf(l[x], e));
+        for (int x = 0; x < OZ_BN; x += 4) {
+          if (i0 + x >= n32) continue;
+          float hi[4], lo[4];
+#pragma unroll
+          for (int y = 0; y < 4; ++y) {
+            const int i = i0 + x + y;
+            float v = 0.0f;
+            if (i < n) {
+              const int e = w.OzE[sp][i] + eb - 2 * OZ_BETA;
+              const float d = __fsub_rn(i == j ? 1.0f : 0.0f, ldexpf(h[x + y], e));
+              v = __fsub_rn(d, ldexpf(l[x + y], e));
+            }
+            tc::tf32_split(v, hi[y], lo[y]);
           }
+          *reinterpret_cast<float4*>(Rh + i0 + x) = make_float4(hi[0], hi[1], hi[2], hi[3]);
+          *reinterpret_cast<float4*>(Rl + i0 + x) = make_float4(lo[0], lo[1], lo[2], lo[3]);
         }
       }
     }
@@ -514,6 +526,8 @@ __global__ void __launch_bounds__(192, 1) k_refine_oz(Config cfg) {
 // Host side
 // ---------------------------------------------------------------------------
 cudaError_t setup_refine_tc() {
+  const cudaError_t e = setup_correct_tc();
+  if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(k_refine_oz, cudaFuncAttributeMaxDynamicSharedMemorySize, OzLayout::SMEM);
 }
 

@@ -646,6 +646,8 @@ bool encode_update_maps(const WalkerDev& w, int ks, int upd_bn, TmapDev* out) {
     // boxes, the MMA's M side) and A (5 planes, 64-row boxes)
     if (w.OzN[sp] && !encode_2d_f16(m + 8, w.OzN[sp], C, 4 * C, 128u)) return false;
     if (w.OzA[sp] && !encode_2d_f16(m + 9, w.OzA[sp], C, 5 * C, 64u)) return false;
+    // low TF32 plane of R^T in the recompute correction
+    if (w.Ascr[sp] && !encode_2d(m + 10, reinterpret_cast<float*>(w.Ascr[sp]) + C * C, C, C, C * 4, TC_BM)) return false;
   }
   return true;
 }

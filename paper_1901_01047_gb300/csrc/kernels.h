@@ -59,7 +59,10 @@ void launch_gj(const Config& cfg, int mode, int max_n, int* d_sgn, cudaStream_t 
 // the two products (R = I - A N0 in FP64, N1 = N0 + N0 R in FP32), then the
 // drift measurement and the copy of N1 into the other buffer.
 void launch_refine_gemms(const Config& cfg, int max_cap, cudaStream_t st);
-// N1 = N0 + N0 R (FP32), R from either residual.
+// N1 = N0 + N0 R: FP32 for the double-float residual's R, 3xTF32 tcgen05 for
+// the split R^T of the digit planes.
+cudaError_t setup_correct_tc();
+void launch_correct_tc(const Config& cfg, cudaStream_t st);
 void launch_refine_correct(const Config& cfg, int max_cap, cudaStream_t st);
 // The residual R = I - A N0 by exponent-aligned digit slicing on the tensor
 // cores (four kernels).

@@ -201,8 +201,9 @@ struct PoolState {
 // TMA tensor maps per walker and spin: update operands A and B, N of parity 0
 // and 1 (128-row boxes), the candidate tables V and U of the tensor-core
 // extension, N of parity 0 and 1 in 32-row boxes (MN-major operand), the
-// digit planes of the sliced recompute residual (N: 128-row boxes, A: 64).
-constexpr int TMAPS_PER_SPIN = 10;
+// digit planes of the sliced recompute residual (N: 128-row boxes, A: 64), the
+// low plane of R^T of the recompute correction (upper half of Ascr).
+constexpr int TMAPS_PER_SPIN = 11;
 
 // Opaque copy of a TMA tensor map (CUtensorMap: 128 bytes, 64-byte aligned).
 struct alignas(64) TmapDev {
