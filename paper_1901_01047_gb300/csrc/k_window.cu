@@ -1329,6 +1329,26 @@ __global__ void k_loop_control(Config cfg, cudaGraphConditionalHandle handle, Lo
   }
 }
 
+__global__ void k_pending(Config cfg, int has_rec, cudaGraphConditionalHandle h_rec, cudaGraphConditionalHandle h_meas,
+                          LoopState* ls) {
+  int rec = 0, meas = 0;
+  for (int i = threadIdx.x; i < cfg.n_walkers; i += 32) {
+    const WalkerDev& w = cfg.W[i];
+    rec |= w.active && w.recompute_pending;
+    meas |= w.active && w.measure_pending;
+  }
+  rec = __any_sync(0xffffffffu, rec);
+  meas = __any_sync(0xffffffffu, meas);
+  if (threadIdx.x == 0) {
+    if (has_rec) {
+      cudaGraphSetConditional(h_rec, rec ? 1u : 0u);
+      ls->rec_total += rec;
+    }
+    cudaGraphSetConditional(h_meas, meas ? 1u : 0u);
+    ls->meas_total += meas;
+  }
+}
+
 __global__ void k_loop_reset(LoopState* ls, int64_t max_iters) {
   ls->iters = 0;
   ls->max_iters = max_iters;
@@ -1456,6 +1476,11 @@ void launch_add_target(const Config& cfg, int64_t n_sweeps, cudaStream_t st) {
 
 void launch_loop_control(const Config& cfg, cudaGraphConditionalHandle handle, LoopState* ls, cudaStream_t st) {
   k_loop_control<<<1, 256, 0, st>>>(cfg, handle, ls);
+}
+
+void launch_pending(const Config& cfg, bool rec, cudaGraphConditionalHandle h_rec, cudaGraphConditionalHandle h_meas,
+                    LoopState* ls, cudaStream_t st) {
+  k_pending<<<1, 32, 0, st>>>(cfg, rec ? 1 : 0, h_rec, h_meas, ls);
 }
 
 void launch_loop_reset(LoopState* ls, int64_t max_iters, cudaStream_t st) { k_loop_reset<<<1, 1, 0, st>>>(ls, max_iters); }

@@ -184,6 +184,7 @@ struct LoopState {
   int64_t iters;
   int64_t max_iters;
   int64_t total_iters;
+  int64_t rec_total, meas_total;  // windows whose recompute / measurement IF node ran (only grow)
   int32_t timed_out;
   int32_t pad;
 };

@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -86,6 +87,8 @@ struct dca_walker {
   dca::LoopState* h_loop = nullptr;  // pinned copy read at synchronisation points
   dca::PoolState* d_pool = nullptr;  // pooled schedule: sweep target and go flag
   int kernels_per_window = 0;
+  int kernels_recompute = 0, kernels_measure = 0;  // and of the parts in IF nodes, when they run
+  int64_t loop_rec_seen = 0, loop_meas_seen = 0;
   int64_t loop_iters_seen = 0;       // window-loop iterations already counted
   bool timeout_pending = false;      // a window loop hit its bound since the last dca_walker_sync
   bool g0_rejected = false;          // an update_G0 table had a non-finite entry (reported by sync)
@@ -606,6 +609,10 @@ static int pull_records(dca_walker* h) {
     h->loop_iters_seen = h->h_loop->total_iters;
     h->windows_launched += it;
     h->total_launches += it * h->kernels_per_window;
+    h->total_launches += (h->h_loop->rec_total - h->loop_rec_seen) * h->kernels_recompute;
+    h->total_launches += (h->h_loop->meas_total - h->loop_meas_seen) * h->kernels_measure;
+    h->loop_rec_seen = h->h_loop->rec_total;
+    h->loop_meas_seen = h->h_loop->meas_total;
     if (h->h_loop->timed_out) {
       h->timeout_pending = true;
       const int32_t zero = 0;
@@ -697,12 +704,16 @@ static void collect_events(dca_walker* h) {
 // Concurrent branches of the captured window for a batch of W walkers.
 static int window_branches(int W) { return W >= 128 ? 4 : (W >= 32 ? 2 : 1); }
 
-// One window's kernel sequence for the walkers of cfg on stream st.
-static int launch_window_sequence(dca_walker* h, const dca::Config& cfg, cudaStream_t st) {
+// Parts of a window: the submatrix update, the recompute, the measurement.
+enum : unsigned { PART_UPDATE = 1, PART_RECOMPUTE = 2, PART_MEASURE = 4, PART_ALL = 7 };
+
+// Kernel sequence of the given parts of one window, for the walkers of cfg on stream st.
+static int launch_window_sequence(dca_walker* h, const dca::Config& cfg, cudaStream_t st, unsigned parts = PART_ALL) {
   int k = 0;
   for (int i = 0; i < dca::N_WINDOW_GROUPS; ++i) {
     const int g = dca::WINDOW_GROUPS[i];
-    if (dca::is_recompute_group(g) && !has_recompute(h)) continue;
+    const unsigned part = dca::is_recompute_group(g) ? PART_RECOMPUTE : (g == dca::GROUP_MEASURE ? PART_MEASURE : PART_UPDATE);
+    if (!(parts & part) || (part == PART_RECOMPUTE && !has_recompute(h))) continue;
     if (g == dca::GROUP_MEASURE)
       k += dca::launch_measure(cfg, h->max_cap, h->max_nc, st);
     else if (g == dca::GROUP_RECOMPUTE_PRE || g == dca::GROUP_RECOMPUTE || g == dca::GROUP_RECOMPUTE_POST)
@@ -711,6 +722,33 @@ static int launch_window_sequence(dca_walker* h, const dca::Config& cfg, cudaStr
       k += dca::launch_window_group(g, cfg, h->max_cap, st);
   }
   return k;
+}
+
+// An IF node behind everything captured on cap_stream so far (a window body),
+// whose body is the given part of the window, of *kernels kernels.
+static int capture_if(dca_walker* h, const dca::Config& cfg, cudaGraphConditionalHandle handle, unsigned part, int* kernels) {
+  cudaStreamCaptureStatus status;
+  unsigned long long id = 0;
+  cudaGraph_t g = nullptr;
+  const cudaGraphNode_t* deps = nullptr;
+  const cudaGraphEdgeData* edges = nullptr;
+  size_t nd = 0;
+  CK(cudaStreamGetCaptureInfo(h->cap_stream, &status, &id, &g, &deps, &edges, &nd));
+  cudaGraphNodeParams np = {};
+  np.type = cudaGraphNodeTypeConditional;
+  np.conditional.handle = handle;
+  np.conditional.type = cudaGraphCondTypeIf;
+  np.conditional.size = 1;
+  cudaGraphNode_t node;
+  CK(cudaGraphAddNode(&node, g, deps, edges, nd, &np));
+  CK(cudaStreamUpdateCaptureDependencies(h->cap_stream, &node, nullptr, 1, cudaStreamSetCaptureDependencies));
+  if (!h->cap_br[0]) CK(cudaStreamCreateWithFlags(&h->cap_br[0], cudaStreamNonBlocking));
+  CK(cudaStreamBeginCaptureToGraph(h->cap_br[0], np.conditional.phGraph_out[0], nullptr, nullptr, 0,
+                                   cudaStreamCaptureModeRelaxed));
+  *kernels = launch_window_sequence(h, cfg, h->cap_br[0], part);
+  cudaGraph_t captured = nullptr;
+  CK(cudaStreamEndCapture(h->cap_br[0], &captured));
+  return DCA_OK;
 }
 
 // Build the device-side window loop once: an outer graph holding one
@@ -761,7 +799,32 @@ static int build_loop_graph(dca_walker* h) {
       CK(cudaStreamWaitEvent(h->cap_stream, h->ev_join[b], 0));
     }
   } else {
-    k += launch_window_sequence(h, h->cfg, h->cap_stream);
+    // Few walkers whose sweeps take many windows: most windows end no sweep and
+    // recompute nothing, so the eight or so kernels of each of these parts sit in
+    // IF nodes.  A node and its setter cost about as much as three idle kernels:
+    // at 9 windows a sweep (bound 12; one mixed walker of 16 sites) a sweep went
+    // from 3.11 to 2.97 ms, at 4 (bound 6) from 1.47 to 1.45 ms; at 3 (bound 5)
+    // it would go from 1.68 to 1.70 ms, at one (the atom) from 97 to 102 us.
+    double windows = 0.0;  // bound of the mean order, K + beta U Nc / 2 = K cosh gamma, in windows
+    for (const ProblemDev& p : h->h_P)
+      windows = std::max(windows, p.K * 0.5 * (p.expV[0][0] + p.expV[0][1]) / (double)h->ks);
+    if (windows >= 6.0) {
+      const bool rec = has_recompute(h);
+      cudaGraphConditionalHandle h_rec = 0, h_meas = 0;
+      if (rec) CK(cudaGraphConditionalHandleCreate(&h_rec, body, 0u, 0u));
+      CK(cudaGraphConditionalHandleCreate(&h_meas, body, 0u, 0u));
+      k += launch_window_sequence(h, h->cfg, h->cap_stream, PART_UPDATE);
+      dca::launch_pending(h->cfg, rec, h_rec, h_meas, h->d_loop, h->cap_stream);
+      k += 1;
+      if (rec) {
+        const int rc = capture_if(h, h->cfg, h_rec, PART_RECOMPUTE, &h->kernels_recompute);
+        if (rc != DCA_OK) return rc;
+      }
+      const int rc = capture_if(h, h->cfg, h_meas, PART_MEASURE, &h->kernels_measure);
+      if (rc != DCA_OK) return rc;
+    } else {
+      k += launch_window_sequence(h, h->cfg, h->cap_stream);
+    }
   }
   dca::launch_loop_control(h->cfg, handle, h->d_loop, h->cap_stream);
   k += 1;

@@ -1,7 +1,8 @@
 """G(tau) of one measurement against the estimator in numpy on the walker's own
 N, at the edges of the product kernels: every site class (nc <= 8, 16, 36, 64
 in FP32; a power of two or not, <= 16 or more in FP64), tau grids that end
-inside a tile, commensurate (n_tau an even multiple) and not.
+inside a tile, commensurate (n_tau an even multiple) and not, orders above and
+below the 256 vertices of an FP32 item.
 
     G(d, a) = g0(d, tau_a) + (1/Nc) sum_{r', i} g0(r' + d - r_i, tau_a - tau_i) b_i(r'),
     b_i(r') = (e^{V_i} - 1) sum_j N_ij g0(r_j - r', tau_j)
@@ -29,13 +30,14 @@ def _interp(table, d, t, beta):
 
 
 @pytest.mark.parametrize("precision", ["fp64", "mixed"])
-@pytest.mark.parametrize("side,ntm,n_tau", [(1, 16, 512), (2, 100, 1000), (2, 130, 512), (3, 128, 512), (4, 33, 1056),
-                                            (5, 96, 576), (6, 129, 1032), (7, 64, 512)])
-def test_measured_G_equals_the_estimator_on_the_same_N(side, ntm, n_tau, precision):
+@pytest.mark.parametrize("side,beta,ntm,n_tau", [(1, 3.0, 16, 512), (2, 3.0, 100, 1000), (2, 3.0, 130, 512),
+                                                 (3, 3.0, 128, 512), (4, 3.0, 33, 1056), (4, 11.0, 40, 1040),
+                                                 (5, 1.5, 96, 576), (6, 1.5, 129, 1032), (7, 1.5, 64, 512)])
+def test_measured_G_equals_the_estimator_on_the_same_N(side, beta, ntm, n_tau, precision):
     import torch
     from paper_1901_01047_gb300 import walker
     c = inputs.make_cluster(((side, 0), (0, side)))
-    nc, U, beta = side * side, 4.0, 3.0 if side < 5 else 1.5
+    nc, U = side * side, 4.0
     eps = inputs.square_dispersion(c.kpts, 1.0 if nc > 1 else 0.0, 0.0)
     G0 = og0.g0_table(eps, inputs.k_dot_r(c), U / 2, U, beta, n_tau)
     prob = dict(nc=nc, site_sub=c.site_sub, U=U, beta=beta, K=1.0, G0=G0)
