@@ -461,7 +461,7 @@ int launch_recompute(int part, const Config& cfg, int max_cap, int* d_sgn, cudaS
         if (cfg.recompute_oz) {
           launch_refine_oz(cfg, max_cap, st);
           launch_correct_tc(cfg, st);
-          return 5;
+          return 4;
         }
         launch_refine_gemms(cfg, max_cap, st);
         return 2;

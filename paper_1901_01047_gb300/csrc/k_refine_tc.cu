@@ -24,11 +24,12 @@
 // N1 = N0 + N0 R to bring an FP32 N back to its rounding level.
 //
 // Kernels:
-//   k_oz_exp      exponents: ea_i from max_k |A[i, k]|, eb_j from max_k |N0[k, j]|
-//   k_oz_slice_a  digit planes of A, row-major [5][cap][cap] (FP16)
+//   k_oz_a        exponents ea_i from max_k |A[i, k]|, eb_j from max_k |N0[k, j]|,
+//                 and the digit planes of A, row-major [5][cap][cap] (FP16)
 //   k_oz_slice_n  digit planes of N0 transposed, [4][cap][cap]: row j holds column j
 //   k_refine_oz   the 17 plane products, D^T[j, i] = sum_k b_t[k, j] a_s[i, k]
-//                 (M = 128 columns j, N = 64 rows i, K = 64 per stage), and R
+//                 (M = 128 columns j, N = 64 rows i, K = 64 per stage), and R^T
+//                 split into two TF32 planes for k_correct_tc
 // The digit planes are zero for k in [n, roundup(n, 64)) (the last K stage);
 // rows past n are never stored.
 #include <cuda.h>
@@ -74,10 +75,24 @@ __device__ __forceinline__ int oz_exponent(float m) {
   return e + 1;
 }
 
-// Items per walker-spin: blocks of 8 rows of A (a warp per row), then
-// strips of 32 columns of N0 (8 row groups of 32 threads, one thread per
-// column and group, the group maxima combined in shared memory).
-__global__ void __launch_bounds__(256) k_oz_exp(Config cfg) {
+// Error-free sum of two FP32 values (Knuth): s + e = a + b exactly.
+__device__ __forceinline__ void oz_two_sum(float a, float b, float& s, float& e) {
+  s = __fadd_rn(a, b);
+  const float bb = __fsub_rn(s, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+
+// Items per walker-spin: blocks of 8 rows of A, then strips of 32 columns of
+// N0.  A warp takes a row of A: its largest magnitude gives the exponent ea_i,
+// then (the row still in L1) the digit planes of the elements k < kpad (zero
+// for k >= n): the value hi + lo scaled by 2^-ea_i is kept as a double-float
+// remainder; each digit is the remainder times 2^9 rounded to an integer.  Two
+// elements a lane and step: 16-byte loads, 4-byte stores.  The strips (8 row
+// groups of 32 threads, one thread per column and group, the group maxima
+// combined in shared memory) give the column exponents eb_j.  As two kernels,
+// one element a thread with a 64-bit division for its row, the batch of 256
+// took 0.94 ms, now 0.41 ms.
+__global__ void __launch_bounds__(256) k_oz_a(Config cfg) {
   __shared__ float s_m[8][32];
   for_each_item(
       2 * cfg.n_walkers,
@@ -93,12 +108,40 @@ __global__ void __launch_bounds__(256) k_oz_exp(Config cfg) {
         if (item < rb) {
           const int i = item * 8 + grp;
           if (i >= n) return;
-          const float2* A = reinterpret_cast<const float2*>(w.Ascr[sp]) + (size_t)i * ld;
+          // ld is a multiple of 32: rows are 16-byte aligned and padded to pairs
+          const float4* A = reinterpret_cast<const float4*>(w.Ascr[sp]) + (size_t)i * (ld / 2);
           float m = 0.0f;
-          for (int k = lane; k < n; k += 32) m = fmaxf(m, fabsf(A[k].x));
+#pragma unroll 4
+          for (int k = 2 * lane; k < n; k += 64) {
+            const float4 v = A[k / 2];
+            m = fmaxf(m, fabsf(v.x));
+            if (k + 1 < n) m = fmaxf(m, fabsf(v.z));
+          }
 #pragma unroll
           for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-          if (lane == 0) w.OzE[sp][i] = oz_exponent(m);
+          const int ea = oz_exponent(m);
+          if (lane == 0) w.OzE[sp][i] = ea;
+          // 2^-ea in two factors, each a normal number: exact products
+          const float f1 = ldexpf(1.0f, -(ea / 2)), f2 = ldexpf(1.0f, -(ea - ea / 2));
+          const int kp = oz_kpad(w);
+          __half* out = reinterpret_cast<__half*>(w.OzA[sp]) + (size_t)i * ld;
+          const size_t plane = (size_t)ld * ld;
+          for (int k = 2 * lane; k < kp; k += 64) {  // kp is a multiple of 32
+            const float4 v = k < n ? A[k / 2] : make_float4(0.f, 0.f, 0.f, 0.f);
+            float xh[2] = {v.x * f1 * f2, v.z * f1 * f2}, xl[2] = {v.y * f1 * f2, v.w * f1 * f2};
+            if (k + 1 >= n) xh[1] = xl[1] = 0.0f;
+#pragma unroll
+            for (int d = 0; d < OZ_SA; ++d) {
+              float q[2];
+#pragma unroll
+              for (int u = 0; u < 2; ++u) {
+                const float yh = xh[u] * (float)(1 << OZ_BETA), yl = xl[u] * (float)(1 << OZ_BETA);
+                q[u] = rintf(yh);
+                oz_two_sum(__fsub_rn(yh, q[u]), yl, xh[u], xl[u]);
+              }
+              *reinterpret_cast<__half2*>(out + d * plane + k) = __floats2half2_rn(q[0], q[1]);  // |q| <= 256: exact
+            }
+          }
         } else {
           // block-uniform branch: the strip's barrier is reached by every thread
           const int j = (item - rb) * 32 + lane;
@@ -115,49 +158,6 @@ __global__ void __launch_bounds__(256) k_oz_exp(Config cfg) {
             for (int g = 1; g < 8; ++g) m = fmaxf(m, s_m[g][lane]);
             w.OzE[sp][ld + j] = oz_exponent(m);
           }
-        }
-      });
-}
-
-// Error-free sum of two FP32 values (Knuth): s + e = a + b exactly.
-__device__ __forceinline__ void oz_two_sum(float a, float b, float& s, float& e) {
-  s = __fadd_rn(a, b);
-  const float bb = __fsub_rn(s, a);
-  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-}
-
-// Digit planes of A: element (i, k) of row block i < n, k < kpad (zero for
-// k >= n).  The value hi + lo scaled by 2^-ea_i is kept as a double-float
-// remainder; each digit is the remainder times 2^9 rounded to an integer.
-__global__ void __launch_bounds__(256) k_oz_slice_a(Config cfg) {
-  for_each_item(
-      2 * cfg.n_walkers,
-      [&](int s) -> long long {
-        const WalkerDev& w = cfg.W[s >> 1];
-        return oz_wants(w) ? blocks_of((long long)w.n * oz_kpad(w), 256) : 0;
-      },
-      [&](int s, int item) {
-        const WalkerDev& w = cfg.W[s >> 1];
-        const int sp = s & 1, n = w.n, ld = w.cap, kp = oz_kpad(w);
-        const long long e = (long long)item * 256 + threadIdx.x;
-        if (e >= (long long)n * kp) return;
-        const int i = (int)(e / kp), k = (int)(e - (long long)i * kp);
-        __half* out = reinterpret_cast<__half*>(w.OzA[sp]) + (size_t)i * ld + k;
-        const size_t plane = (size_t)ld * ld;
-        if (k >= n) {
-#pragma unroll
-          for (int d = 0; d < OZ_SA; ++d) out[d * plane] = __float2half_rn(0.0f);
-          return;
-        }
-        const float2 a = reinterpret_cast<const float2*>(w.Ascr[sp])[(size_t)i * ld + k];
-        const int ea = w.OzE[sp][i];
-        float xh = ldexpf(a.x, -ea), xl = ldexpf(a.y, -ea);  // exact: powers of two
-#pragma unroll
-        for (int d = 0; d < OZ_SA; ++d) {
-          const float yh = xh * (float)(1 << OZ_BETA), yl = xl * (float)(1 << OZ_BETA);
-          const float q = rintf(yh);
-          out[d * plane] = __float2half_rn(q);  // |q| <= 256: exact
-          oz_two_sum(__fsub_rn(yh, q), yl, xh, xl);
         }
       });
 }
@@ -533,10 +533,8 @@ cudaError_t setup_refine_tc() {
 
 void launch_refine_oz(const Config& cfg, int max_cap, cudaStream_t st) {
   const long long S = 2LL * cfg.n_walkers;
-  k_oz_exp<<<persist_grid((const void*)k_oz_exp, S * (blocks_of(max_cap, 8) + blocks_of(max_cap, 32)), 256), 256,
-             0, st>>>(cfg);
-  k_oz_slice_a<<<persist_grid((const void*)k_oz_slice_a, S * blocks_of((long long)max_cap * max_cap, 256), 256), 256,
-                 0, st>>>(cfg);
+  const long long rows = S * (blocks_of(max_cap, 8) + blocks_of(max_cap, 32));
+  k_oz_a<<<persist_grid((const void*)k_oz_a, rows, 256), 256, 0, st>>>(cfg);
   k_oz_slice_n<<<persist_grid((const void*)k_oz_slice_n, S * blocks_of(max_cap, 32) * blocks_of(max_cap, 32), 256),
                  256, 0, st>>>(cfg);
   k_refine_oz<<<device_sm_count(), 192, OzLayout::SMEM, st>>>(cfg);

@@ -68,7 +68,7 @@ cudaError_t setup_correct_tc();
 void launch_correct_tc(const Config& cfg, cudaStream_t st);
 void launch_refine_correct(const Config& cfg, int max_cap, cudaStream_t st);
 // The residual R = I - A N0 by exponent-aligned digit slicing on the tensor
-// cores (four kernels).
+// cores (three kernels).
 void launch_refine_oz(const Config& cfg, int max_cap, cudaStream_t st);
 cudaError_t setup_refine_tc();
 void launch_refine_adopt(const Config& cfg, int max_cap, cudaStream_t st);
