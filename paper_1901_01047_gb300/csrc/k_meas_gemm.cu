@@ -18,6 +18,14 @@ namespace {
 constexpr int MK = 32;    // vertices per tile
 constexpr int MT = 128;   // tau points per item, FP32 kernel
 constexpr int AST = MT + 4;
+// Vertices per item of the FP32 kernel for up to 16 sites: a window measures a
+// few walkers only, and one of 16 sites with 256 tau points is 64 items without
+// this split (a measurement of 16 sites, order 640, 114 -> 76 us).  Larger clusters
+// have items enough, and the split costs 4 of 36 sites 7 % of a sweep.
+template <int CLASS>
+__host__ __device__ constexpr int vseg() {
+  return CLASS == 0 ? 256 : 1 << 30;
+}
 constexpr int DT = 16;    // tau points per item, FP64 kernel
 
 __device__ __forceinline__ bool wants_gemm(const WalkerDev& w) { return w.active && w.measure_pending; }
@@ -70,7 +78,7 @@ __device__ __forceinline__ void df_add(float& hi, float& lo, float x) {
   hi = s;
 }
 
-template <int NG, int SR, int TA>
+template <int CLASS, int NG, int SR, int TA>
 __device__ __forceinline__ void meas_item_f(const Config& cfg, const WalkerDev& w, int sp, int item, MeasSmem& sm,
                                             float* dyn) {
   constexpr int TT = MT / TA;            // tau threads
@@ -80,8 +88,11 @@ __device__ __forceinline__ void meas_item_f(const Config& cfg, const WalkerDev& 
   constexpr int PAD = (SR + 3) & ~3;
   constexpr int BST = bs_stride<NG, SR>();
   const ProblemDev& pb = cfg.P[w.problem];
-  const int nc = pb.nc, ntm = cfg.n_tau_meas, n = w.n, par = w.parity, ld = w.cap, q = pb.meas_q;
-  const int tblocks = (ntm + MT - 1) / MT;
+  const int nc = pb.nc, ntm = cfg.n_tau_meas, par = w.parity, ld = w.cap, q = pb.meas_q;
+  constexpr int VS = vseg<CLASS>();
+  const int tblocks = (ntm + MT - 1) / MT, segs = (int)blocks_of(w.n, VS);
+  const int v0 = (item % segs) * VS, n = (int)min((long long)w.n, (long long)v0 + VS);  // the item's vertices v0 .. n - 1
+  item /= segs;
   const int x = item / tblocks, a0 = (item - x * tblocks) * MT;
   const int tid = threadIdx.x, kg = tid / TPG, tg = tid - kg * TPG, sg = tg / TT, ta = tg - sg * TT;
   float* const As = dyn;                      // [2][MK][AST]
@@ -204,14 +215,14 @@ __device__ __forceinline__ void meas_item_f(const Config& cfg, const WalkerDev& 
   };
 
   __syncthreads();  // the previous item of this block is done with the shared tiles
-  if (n > 0) {
-    prep(0, 0);
-    if (MK < n) prep(MK, 1);
+  if (v0 < n) {
+    prep(v0, 0);
+    if (v0 + MK < n) prep(v0 + MK, 1);
     __syncthreads();
     fetch(0);
-    fill(0, 0);
+    fill(v0, 0);
     __syncthreads();
-    for (int i0 = 0, t = 0; i0 < n; i0 += MK, ++t) {
+    for (int i0 = v0, t = 0; i0 < n; i0 += MK, ++t) {
       const int b = t & 1;
       if (i0 + MK < n) fetch(b ^ 1);
       compute(b);
@@ -270,17 +281,18 @@ __global__ void __launch_bounds__(256, CLASS == 2 ? 1 : 2) k_meas_gemm(Config cf
       [&](int s) -> long long {
         const WalkerDev& w = cfg.W[s >> 1];
         const int nc = cfg.P[w.problem].nc;
-        return (wants_gemm(w) && site_class(nc) == CLASS) ? (long long)nc * blocks_of(cfg.n_tau_meas, MT) : 0;
+        return (wants_gemm(w) && site_class(nc) == CLASS)
+                   ? (long long)nc * blocks_of(cfg.n_tau_meas, MT) * blocks_of(w.n, vseg<CLASS>()) : 0;
       },
       [&](int s, int item) {
         const WalkerDev& w = cfg.W[s >> 1];
         if constexpr (CLASS == 0) {
-          if (cfg.P[w.problem].nc <= 8) meas_item_f<2, 4, 4>(cfg, w, s & 1, item, sm, dyn);
-          else meas_item_f<4, 4, 4>(cfg, w, s & 1, item, sm, dyn);
+          if (cfg.P[w.problem].nc <= 8) meas_item_f<CLASS, 2, 4, 4>(cfg, w, s & 1, item, sm, dyn);
+          else meas_item_f<CLASS, 4, 4, 4>(cfg, w, s & 1, item, sm, dyn);
         } else if constexpr (CLASS == 1) {
-          meas_item_f<4, 9, 2>(cfg, w, s & 1, item, sm, dyn);
+          meas_item_f<CLASS, 4, 9, 2>(cfg, w, s & 1, item, sm, dyn);
         } else {
-          meas_item_f<4, 16, 2>(cfg, w, s & 1, item, sm, dyn);
+          meas_item_f<CLASS, 4, 16, 2>(cfg, w, s & 1, item, sm, dyn);
         }
       });
 }
@@ -405,11 +417,11 @@ static void gemm_f(const Config& cfg, long long items, cudaStream_t st) {
   k_meas_gemm<CLASS><<<persist_grid((const void*)k_meas_gemm<CLASS>, items, 256, sm), 256, sm, st>>>(cfg);
 }
 
-int launch_meas_gemm(const Config& cfg, int max_nc, cudaStream_t st) {
+int launch_meas_gemm(const Config& cfg, int max_cap, int max_nc, cudaStream_t st) {
   const long long S = 2LL * cfg.n_walkers;
   if (cfg.prec == PREC_MIXED) {
     const long long items = S * max_nc * blocks_of(cfg.n_tau_meas, MT);
-    gemm_f<0>(cfg, items, st);
+    gemm_f<0>(cfg, items * blocks_of(max_cap, vseg<0>()), st);
     if (max_nc > 16) gemm_f<1>(cfg, items, st);
     if (max_nc > 36) gemm_f<2>(cfg, items, st);
     return 1 + (max_nc > 16) + (max_nc > 36);

@@ -76,7 +76,7 @@ void launch_refine_adopt(const Config& cfg, int max_cap, cudaStream_t st);
 int launch_recompute(int part, const Config& cfg, int max_cap, int* d_sgn, cudaStream_t st);
 // The product of a measurement (k_meas_gemm.cu); returns the number of kernels.
 cudaError_t setup_meas_gemm();
-int launch_meas_gemm(const Config& cfg, int max_nc, cudaStream_t st);
+int launch_meas_gemm(const Config& cfg, int max_cap, int max_nc, cudaStream_t st);
 int launch_measure(const Config& cfg, int max_cap, int max_nc, cudaStream_t st);
 
 // Streaming multiprocessors of the current device (queried once per device;
