@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(192, 1) k_upd_tc(Config cfg) {
 // the candidate columns G_ext[x < n, c] are FP32 products, so exact in FP32;
 // the per-column factors e^{V} / (e^{V} - 1) a_p are formed once per item in
 // FP64 and split), in FP64 for the rows of accepted insertions (X is FP64).
-// Items per walker-spin: ceil(rows / 32) row blocks (rows = n + n_ins), then
+// Items per walker-spin: row blocks of fact_rows(l) of the n + n_ins rows, then
 // ceil(n / 32) column blocks.  Dynamic shared memory: the L rows of a row
 // block [32][ld], ld = 65 with k_s <= 64 (then also B^-1, [64][64]) or 129
 // (odd strides: the rows a warp reads at one p fall in different banks); a
@@ -355,6 +355,13 @@ constexpr int FACT_RB = 32, FACT_BS = 64, FACT_PB = 8;
 __host__ __device__ constexpr size_t fact_smem(bool bs) {
   return bs ? sizeof(float2) * (FACT_RB * (FACT_BS + 1) + FACT_BS * FACT_BS) : sizeof(float2) * FACT_RB * (KS_MAX + 1);
 }
+
+// Rows of a row block: as many groups of four outputs as the block has threads
+// (28 rows at l = 33 to 36), so that L' takes one full pass; with 32 rows and
+// the padding to lpad = 64 dealt out as well, the two passes of l a little above
+// 32, the usual case of 64 proposals, left almost half the lanes of these
+// 13-instruction steps idle.  256 walkers, 64 proposals: 434 -> 384 us a window.
+__device__ __forceinline__ int fact_rows(int l) { return min(FACT_RB, 256 / ((l + 3) / 4)); }
 
 __global__ void __launch_bounds__(256) k_upd_factors(Config cfg) {
   constexpr int RB = FACT_RB;
@@ -372,20 +379,20 @@ __global__ void __launch_bounds__(256) k_upd_factors(Config cfg) {
       [&](int s) -> long long {
         const WalkerDev& w = cfg.W[s >> 1];
         if (!(w.active && w.n_acc > 0)) return 0;
-        return blocks_of(w.n + w.n_ins, RB) + blocks_of(w.n, RB);
+        return blocks_of(w.n + w.n_ins, fact_rows(w.n_acc)) + blocks_of(w.n, RB);
       },
       [&](int s, int item) {
         const WalkerDev& w = cfg.W[s >> 1];
         const int sp = s & 1, n = w.n, l = w.n_acc, cap = w.cap, ld = w.cap;
         const int rows = n + w.n_ins, lpad = (l + 31) & ~31;
-        const int ra = (int)blocks_of(rows, RB);
+        const int rb = fact_rows(l), ra = (int)blocks_of(rows, rb);
         const ProblemDev& pb = cfg.P[w.problem];
         const float* N = (const float*)w.N[w.parity][sp];
         const int* vs = w.vs[w.parity];
         __syncthreads();  // the previous item is done with the shared tiles
         if (item < ra) {
-          const int t0 = item * RB;
-          for (int r = threadIdx.x; r < RB; r += blockDim.x) {
+          const int t0 = item * rb;
+          for (int r = threadIdx.x; r < rb; r += blockDim.x) {
             const int t = t0 + r;
             int x = -1;
             if (t < rows) {
@@ -415,13 +422,13 @@ __global__ void __launch_bounds__(256) k_upd_factors(Config cfg) {
           __syncthreads();
           // L in batches of FACT_PB entries per thread: the loads of a batch are all
           // issued before the arithmetic (they are scattered columns of N)
-          for (int e0 = 0; e0 < RB * l; e0 += FACT_PB * 256) {
+          for (int e0 = 0; e0 < rb * l; e0 += FACT_PB * 256) {
             float gv[FACT_PB];
 #pragma unroll
             for (int k = 0; k < FACT_PB; ++k) {
               const int e = e0 + k * 256 + threadIdx.x;
               gv[k] = 0.f;
-              if (e < RB * l) {
+              if (e < rb * l) {
                 const int r = e / l, p = e - r * l;
                 const int x = s_xr[r], P = s_pp[p];
                 if (x >= 0 && x < n && s_ok[p])
@@ -431,7 +438,7 @@ __global__ void __launch_bounds__(256) k_upd_factors(Config cfg) {
 #pragma unroll
             for (int k = 0; k < FACT_PB; ++k) {
               const int e = e0 + k * 256 + threadIdx.x;
-              if (e >= RB * l) break;
+              if (e >= rb * l) break;
               const int r = e / l, p = e - r * l;
               const int x = s_xr[r], P = s_pp[p];
               float2 v = make_float2(0.f, 0.f);
@@ -463,23 +470,22 @@ __global__ void __launch_bounds__(256) k_upd_factors(Config cfg) {
           }
           __syncthreads();
           // L' = L B^-1: four consecutive outputs of a row per thread (four
-          // independent double-float chains sharing the loads of L)
-          const int lq = lpad / 4;
-          for (int e = threadIdx.x; e < RB * lq; e += blockDim.x) {
+          // independent double-float chains sharing the loads of L), the groups
+          // that start below l
+          const int lq = (l + 3) / 4;
+          for (int e = threadIdx.x; e < rb * lq; e += blockDim.x) {
             const int r = e / lq, q = (e - r * lq) * 4;
             const int t = t0 + r;
             if (t >= rows) continue;
             const int x = t < n ? t : n + w.acc_slot[t - n];
             float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
-            if (q < l) {
-              for (int p = 0; p < l; ++p) {
-                const float2 a = s_Lb[r * lds + p];
-                const float2* brow = bs ? s_binv + p * FACT_BS + q : Bi + (size_t)p * KS_MAX + q;
+            for (int p = 0; p < l; ++p) {
+              const float2 a = s_Lb[r * lds + p];
+              const float2* brow = bs ? s_binv + p * FACT_BS + q : Bi + (size_t)p * KS_MAX + q;
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                  const float2 b = brow[u];  // columns >= l of B^-1 are never read back
-                  df_fma(hi[u], lo[u], a.x, a.y, b.x, b.y);
-                }
+              for (int u = 0; u < 4; ++u) {
+                const float2 b = brow[u];  // columns >= l of B^-1 are never read back
+                df_fma(hi[u], lo[u], a.x, a.y, b.x, b.y);
               }
             }
             float2* lp = reinterpret_cast<float2*>(w.Lp[sp]) + (size_t)x * KS_MAX + q;
@@ -494,6 +500,14 @@ __global__ void __launch_bounds__(256) k_upd_factors(Config cfg) {
                 w.Aop[sp][((size_t)cap + x) * TC_KS + q + u] = tl;
               }
             }
+          }
+          // zeros of the operand from there to lpad
+          const int zq = lpad / 4 - lq;
+          for (int e = threadIdx.x; e < rb * zq; e += blockDim.x) {
+            const int r = e / zq, q = (lq + e - r * zq) * 4, x = t0 + r;
+            if (x >= n) continue;
+            *reinterpret_cast<float4*>(w.Aop[sp] + (size_t)x * TC_KS + q) = make_float4(0.f, 0.f, 0.f, 0.f);
+            *reinterpret_cast<float4*>(w.Aop[sp] + ((size_t)cap + x) * TC_KS + q) = make_float4(0.f, 0.f, 0.f, 0.f);
           }
         } else {
           // R rows (Rr, for the border update) and the transposed split B operand
@@ -534,7 +548,7 @@ __global__ void __launch_bounds__(256) k_upd_factors(Config cfg) {
 }
 
 void launch_upd_factors(const Config& cfg, int max_cap, cudaStream_t st) {
-  const long long items = 2LL * cfg.n_walkers * (blocks_of(max_cap, 32) + blocks_of(max_cap, 32));
+  const long long items = 2LL * cfg.n_walkers * (blocks_of(max_cap, 16) + blocks_of(max_cap, 32));
   const size_t smem = fact_smem(cfg.ks <= FACT_BS);
   k_upd_factors<<<persist_grid((const void*)k_upd_factors, items, 256, smem), 256, smem, st>>>(cfg);
 }
