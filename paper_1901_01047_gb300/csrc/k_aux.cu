@@ -504,10 +504,11 @@ void launch_rebuild(const Config& cfg, int max_n, int* d_sgn, cudaStream_t st) {
 
 // From-scratch N for the vertex list held in the current buffer of every walker
 // of cfg (used by the standalone fresh-N operations): build A, invert in place.
-void launch_fresh_inverse(const Config& cfg, int max_n, int* d_sgn, cudaStream_t st) {
+void launch_fresh_inverse(const Config& cfg, int max_n, int* d_sgn, cudaStream_t st, bool wide) {
   const int W = cfg.n_walkers;
   if (max_n <= 0) return;
   k_build_A<<<grid_for(2LL * W * blocks_of((long long)max_n * max_n, 256)), 256, 0, st>>>(cfg, 0);
+  if (wide && launch_gj_wide(cfg, max_n, d_sgn, st)) return;
   launch_gj(cfg, 0, max_n, d_sgn, st);
 }
 

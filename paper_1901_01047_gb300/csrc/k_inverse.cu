@@ -76,9 +76,12 @@ __host__ __device__ __forceinline__ size_t gj_work_bytes(int rows, int B) {
   return sizeof(double) * ((size_t)rows * (B + 1) + (size_t)B * GJ_XC);
 }
 
-template <int B>
+// The whole inverse of one matrix (ONE = false), or (ONE) steps 1 and 2 of the
+// panel at `first`: the panel factors then go to the scratch at 16 n for
+// k_gj_update, the permutation is kept at 32 n for k_gj_finish.
+template <int B, bool ONE>
 __device__ void gj_matrix(const Config& cfg, int mode, int mat, int* sgn_out, cg::cluster_group& cluster, int max_n,
-                          size_t work_bytes) {
+                          size_t work_bytes, int first = 0) {
   const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   const int wi = mat >> 1, sp = mat & 1;
   WalkerDev& w = cfg.W[wi];
@@ -88,8 +91,10 @@ __device__ void gj_matrix(const Config& cfg, int mode, int mat, int* sgn_out, cg
   extern __shared__ __align__(16) unsigned char gj_smem[];
   // rp [n]: original row now at each position; in shared memory with panels of
   // 16, else one copy per block behind the first 8 rows of the scratch
-  int* rp = B == 16 ? reinterpret_cast<int*>(gj_smem) : reinterpret_cast<int*>(X + 8 * (size_t)n) + (size_t)rank * n;
-  double* pan = reinterpret_cast<double*>(gj_smem + gj_rp_bytes(max_n, B));
+  int* rp = ONE ? reinterpret_cast<int*>(X + 32 * (size_t)n)
+                : (B == 16 ? reinterpret_cast<int*>(gj_smem)
+                           : reinterpret_cast<int*>(X + 8 * (size_t)n) + (size_t)rank * n);
+  double* pan = reinterpret_cast<double*>(gj_smem + (ONE ? 0 : gj_rp_bytes(max_n, B)));
   const int rows = n > rank ? (n - rank + C - 1) / C : 0;  // own rows rank, rank + C, ...
   double* xs = pan + (size_t)gj_rows(max_n, C) * (B + 1);
   constexpr int PS = B + 1;
@@ -104,9 +109,11 @@ __device__ void gj_matrix(const Config& cfg, int mode, int mat, int* sgn_out, cg
   constexpr unsigned FULL = 0xffffffffu;
   int sign = 1;
   bool bad = false;
-  for (int i = tid; i < n; i += GJ_THREADS) rp[i] = i;
+  if (ONE && first > 0 && sgn_out[mat] == 0) return;  // an earlier panel was singular (read before any barrier)
+  if (!ONE || (first == 0 && rank == 0))
+    for (int i = tid; i < n; i += GJ_THREADS) rp[i] = i;
 
-  for (int c0 = 0; c0 < n && !bad; c0 += B) {
+  for (int c0 = first; c0 < n && !bad; c0 += B) {
     const int b = min(B, n - c0);
     __syncthreads();  // the own rows are up to date, the shared panel and X are free
     for (int e = tid; e < rows * B; e += GJ_THREADS) {
@@ -199,9 +206,11 @@ __device__ void gj_matrix(const Config& cfg, int mode, int mat, int* sgn_out, cg
             s_d = d;
             s_p = idx;
             s_piv[s] = idx;
-            const int t = rp[c];
-            rp[c] = rp[idx];
-            rp[idx] = t;
+            if (!ONE || rank == 0) {
+              const int t = rp[c];
+              rp[c] = rp[idx];
+              rp[idx] = t;
+            }
           }
         }
         if (lane == 0) s_bad = m > 0ull ? 0 : 1;
@@ -267,7 +276,18 @@ __device__ void gj_matrix(const Config& cfg, int mode, int mat, int* sgn_out, cg
         else A[(size_t)s_dst[warp] * ld + k] = v;
       }
     }
+    if constexpr (ONE) {
+      double* P = X + 16 * (size_t)n;
+      for (int e = tid; e < rows * B; e += GJ_THREADS) {
+        const int r = e / B, j = e - r * B;
+        P[(size_t)(rank + r * C) * B + j] = pan[r * PS + j];
+      }
+    }
     cluster.sync();
+    if constexpr (ONE) {
+      if (rank == 0 && tid == 0) sgn_out[mat] = first == 0 ? sign : sign * sgn_out[mat];
+      return;
+    }
     // update of the own rows
     for (int kb = 0; kb < n; kb += GJ_XC) {
       const int m = min(GJ_XC, n - kb);
@@ -359,9 +379,76 @@ __global__ void __launch_bounds__(GJ_THREADS) k_gj_cluster(Config cfg, int mode,
     cluster.sync();  // every block has read s_next before it changes
     if (mat >= 2 * cfg.n_walkers) break;
     if (!gj_wants(cfg, mode, mat)) continue;
-    gj_matrix<B>(cfg, mode, mat, sgn_out, cluster, max_n, work_bytes);
+    gj_matrix<B, false>(cfg, mode, mat, sgn_out, cluster, max_n, work_bytes);
     cluster.sync();  // the next matrix reuses the shared posts and pivots
   }
+}
+
+// One matrix over the whole device, a kernel pair per panel (n known to the
+// host): the panel's factors on one cluster, then the update of everything else
+// by all SMs.  With the update on the cluster's 16 SMs as well, n^3 multiply-adds
+// on 32 a cycle took half the time: dca_fresh_N of order 500 4.33 -> 3.21 ms.  At
+// order 256 the two launches a panel still cost what the update saves (1.59 ms
+// against 1.52 on the cluster), hence GW_MIN.
+constexpr int GW_B = 16, GW_R = 8, GW_C = 64;  // panel; rows and columns of an update item
+constexpr int GW_MIN = 320, GW_MAX = 4096;     // orders that take this path
+
+__global__ void __launch_bounds__(GJ_THREADS) k_gj_panel(Config cfg, int first, int max_n, int* sgn_out) {
+  cg::cluster_group cluster = cg::this_cluster();
+  const int mat = blockIdx.x / (int)cluster.num_blocks();
+  gj_matrix<GW_B, true>(cfg, 0, mat, sgn_out, cluster, max_n, 0, first);
+}
+
+__global__ void __launch_bounds__(256) k_gj_update(Config cfg, int c0, const int* sgn) {
+  __shared__ double xs[GW_B][GW_C], ps[GW_R][GW_B];
+  const int tid = threadIdx.x, k = tid & (GW_C - 1), rg = tid / GW_C;
+  for_each_item(
+      2 * cfg.n_walkers,
+      [&](int s) -> long long {
+        const int n = cfg.W[s >> 1].n;
+        return c0 < n && sgn[s] != 0 ? blocks_of(n, GW_R) * blocks_of(n, GW_C) : 0;
+      },
+      [&](int s, int item) {
+        const WalkerDev& w = cfg.W[s >> 1];
+        const int sp = s & 1, n = w.n, ld = w.cap, b = min(GW_B, n - c0), cblocks = (n + GW_C - 1) / GW_C;
+        const int i0 = (item / cblocks) * GW_R, k0 = (item % cblocks) * GW_C, col = k0 + k;
+        double* A = cfg.prec == PREC_MIXED ? w.Ascr[sp] : (double*)w.N[w.parity][sp];
+        const double* X = w.Lrow[sp];
+        const double* P = X + 16 * (size_t)n;
+        __syncthreads();  // the previous item is done with the shared tiles
+        for (int e = tid; e < GW_B * GW_C; e += 256) {
+          const int j = e / GW_C, c = k0 + (e - j * GW_C);
+          xs[j][e - j * GW_C] = (j < b && c < n && (c < c0 || c >= c0 + b)) ? X[(size_t)j * n + c] : 0.0;
+        }
+        if (tid < GW_R * GW_B) ps[tid / GW_B][tid % GW_B] = i0 + tid / GW_B < n ? P[(size_t)i0 * GW_B + tid] : 0.0;
+        __syncthreads();
+        if (col >= n) return;
+        const bool in_panel = col >= c0 && col < c0 + b;
+#pragma unroll
+        for (int u = 0; u < GW_R / 4; ++u) {
+          const int r = rg + 4 * u, i = i0 + r;
+          if (i >= n) break;
+          double* a = A + (size_t)i * ld + col;
+          double v = (i >= c0 && i < c0 + b) ? 0.0 : *a;
+#pragma unroll
+          for (int j = 0; j < GW_B; ++j) v = fma(ps[r][j], xs[j][k], v);
+          *a = in_panel ? ps[r][col - c0] : v;
+        }
+      });
+}
+
+// The interchanges undone: column rp[k] of the inverse is the working column k;
+// one block per row.
+__global__ void __launch_bounds__(256) k_gj_finish(Config cfg, const int* sgn) {
+  extern __shared__ double row[];
+  const int mat = blockIdx.y, sp = mat & 1, i = blockIdx.x;
+  const WalkerDev& w = cfg.W[mat >> 1];
+  if (i >= w.n || sgn[mat] == 0) return;
+  const int* rp = reinterpret_cast<const int*>(w.Lrow[sp] + 32 * (size_t)w.n);
+  double* A = (cfg.prec == PREC_MIXED ? w.Ascr[sp] : (double*)w.N[w.parity][sp]) + (size_t)i * w.cap;
+  for (int k = threadIdx.x; k < w.n; k += blockDim.x) row[k] = A[k];
+  __syncthreads();
+  for (int k = threadIdx.x; k < w.n; k += blockDim.x) A[rp[k]] = row[k];
 }
 
 template <int B>
@@ -414,7 +501,64 @@ bool gj_setup() {
   return got > 0;
 }
 
+size_t gw_smem(int n) { return sizeof(double) * (size_t)gj_rows(n, GJ_MAX_CTAS) * (GW_B + 1); }
+
+cudaLaunchConfig_t gw_config(int n, int mats, cudaLaunchAttribute* at, cudaStream_t st) {
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3(GJ_MAX_CTAS * mats);
+  lc.blockDim = dim3(GJ_THREADS);
+  lc.dynamicSmemBytes = gw_smem(n);
+  lc.stream = st;
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = GJ_MAX_CTAS;
+  at->val.clusterDim.y = 1;
+  at->val.clusterDim.z = 1;
+  lc.attrs = at;
+  lc.numAttrs = 1;
+  return lc;
+}
+
+// Whether clusters of 16 blocks of the panel kernel fit the device.
+bool gw_setup() {
+  cudaFuncSetAttribute(k_gj_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gw_smem(GW_MAX));
+  int got = 0;
+  cudaLaunchAttribute at;
+  const cudaLaunchConfig_t lc = gw_config(GW_MAX, 1, &at, nullptr);
+  if (cudaFuncSetAttribute(k_gj_panel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&got, k_gj_panel, &lc) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return got > 0;
+}
+
 }  // namespace
+
+size_t gj_wide_scratch(int n) { return sizeof(double) * 33 * (size_t)n; }
+
+bool launch_gj_wide(const Config& cfg, int n, int* d_sgn, cudaStream_t st) {
+  static std::mutex mu;
+  static int state[64] = {0};  // per device: 0 unknown, 1 not available, 2 available
+  if (n < GW_MIN || n > GW_MAX) return false;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+  {
+    std::lock_guard<std::mutex> lk(mu);
+    if (state[dev] == 0) state[dev] = gw_setup() ? 2 : 1;
+    if (state[dev] != 2) return false;
+  }
+  const int mats = 2 * cfg.n_walkers;
+  const long long items = (long long)mats * blocks_of(n, GW_R) * blocks_of(n, GW_C);
+  const int grid = persist_grid((const void*)k_gj_update, items, 256);
+  cudaLaunchAttribute at;
+  const cudaLaunchConfig_t lc = gw_config(n, mats, &at, st);
+  for (int c0 = 0; c0 < n; c0 += GW_B) {
+    cudaLaunchKernelEx(&lc, k_gj_panel, cfg, c0, n, d_sgn);
+    k_gj_update<<<grid, 256, 0, st>>>(cfg, c0, d_sgn);
+  }
+  k_gj_finish<<<dim3(n, mats), 256, sizeof(double) * n, st>>>(cfg, d_sgn);
+  return true;
+}
 
 void launch_gj(const Config& cfg, int mode, int max_n, int* d_sgn, cudaStream_t st) {
   static std::mutex mu;

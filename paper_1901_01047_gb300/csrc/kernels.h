@@ -55,7 +55,12 @@ void launch_init(const Config& cfg, int n0, int max_cap, int* d_sgn, cudaStream_
 // N of every walker from scratch for the vertex list of its current buffer
 // (live rows 0 .. n-1), and the configuration sign.
 void launch_rebuild(const Config& cfg, int max_n, int* d_sgn, cudaStream_t st);
-void launch_fresh_inverse(const Config& cfg, int max_n, int* d_sgn, cudaStream_t st);
+void launch_fresh_inverse(const Config& cfg, int max_n, int* d_sgn, cudaStream_t st, bool wide = false);
+// The inverse spread over the whole device, for matrices of order n that all
+// walkers share (dca_fresh_N) with gj_wide_scratch(n) bytes behind Lrow; false
+// (nothing launched) where the order or the device is better served by launch_gj.
+size_t gj_wide_scratch(int n);
+bool launch_gj_wide(const Config& cfg, int n, int* d_sgn, cudaStream_t st);
 // Gauss-Jordan inverse of the FP64 work matrices, one 8-block cluster each.
 void launch_gj(const Config& cfg, int mode, int max_n, int* d_sgn, cudaStream_t st);
 // Mixed-precision recompute by one Newton step against the FP64 A = N^-1:

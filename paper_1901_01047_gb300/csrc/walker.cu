@@ -1616,7 +1616,7 @@ extern "C" DCA_API int dca_fresh_N(const dca_problem* problem, int32_t n, const 
                                {(void**)&d_W, sizeof(WalkerDev)},          {(void**)&d_site, sizeof(int32_t) * n},
                                {(void**)&d_tau, sizeof(double) * n},       {(void**)&d_s, sizeof(int32_t) * n},
                                {(void**)&d_N[0], sizeof(double) * nn},     {(void**)&d_N[1], sizeof(double) * nn},
-                               {(void**)&d_scr[0], sizeof(double) * 16 * n}, {(void**)&d_scr[1], sizeof(double) * 16 * n},
+                               {(void**)&d_scr[0], dca::gj_wide_scratch(n)}, {(void**)&d_scr[1], dca::gj_wide_scratch(n)},
                                {(void**)&d_sgn, sizeof(int32_t) * 4}};
   size_t total = 0;
   for (auto& pc : pieces) total += align_up(pc.bytes, 256);
@@ -1666,7 +1666,7 @@ extern "C" DCA_API int dca_fresh_N(const dca_problem* problem, int32_t n, const 
   if (e == cudaSuccess) e = cudaMemcpy(d_tau, tau.data(), sizeof(double) * n, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(d_s, s.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) {
-    dca::launch_fresh_inverse(cfg, n, d_sgn, nullptr);
+    dca::launch_fresh_inverse(cfg, n, d_sgn, nullptr, true);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaMemcpy(sgn, d_sgn, sizeof(sgn), cudaMemcpyDeviceToHost);
