@@ -3,7 +3,8 @@
 // N^-1 = A = e^V - g0 (e^V - 1) of the current configuration (Eq. Zk), which
 // k_build_A forms in FP64 and stores as FP32 pairs (hi, lo):
 //     R  = I - A N0      FP64-grade (double-float products and sums)
-//     N1 = N0 + N0 R     FP32 (R is of the size of the drift)
+//     N1 = N0 + N0 R     FP32 (R is of the size of the drift; with the residual
+//                        from digit planes 3xTF32, k_correct_tc.cu)
 // One step squares the relative error of N0: an FP32 N0 that drifted by 1e-5
 // comes back to the FP32 rounding level.  Both products are tiled GEMMs on a
 // persistent grid over (walker-spin, 64 x 64 output tile), so one walker's

@@ -915,71 +915,59 @@ __device__ __forceinline__ double lp_pair_value(const double* Lp, size_t i) {
 // Extended row of the t-th row of the update (existing rows first).
 __device__ __forceinline__ int upd_row(const WalkerDev& w, int t) { return t < w.n ? t : w.n + w.acc_slot[t - w.n]; }
 
-// Lrow[x, p] = (G_ext[x, P_p] - delta) a_p ; grid = (row blocks, walkers*2), block 256
-template <typename T>
-__global__ void __launch_bounds__(256) k_upd_lrow(Config cfg) {
-  for_each_item(
-      2 * cfg.n_walkers,
-      [&](int s) -> long long {
-        const WalkerDev& w = cfg.W[s >> 1];
-        return upd_active(w) ? blocks_of((long long)(w.n + w.n_ins) * w.n_acc, 256) : 0;
-      },
-      [&](int s, int item) {
-  const WalkerDev& w = cfg.W[s >> 1];
-  const int sp = s & 1;
-  const ProblemDev& pb = cfg.P[w.problem];
-  const int l = w.n_acc, rows = w.n + w.n_ins;
-  const ExtView<T> v = make_view<T>(w, sp);
-  const int total = rows * l;
-  const int idx = item * 256 + threadIdx.x;
-  if (idx < total) {
-    const int t = idx / l, p = idx - t * l;
-    const int x = upd_row(w, t), P = w.P[p];
-    const double a = w.aP[sp][p];
-    double val = 0.0;
-    if (a != 0.0 && !(x < w.n && v.vs[x] == 0)) val = (g_ext(v, pb, sp, x, P) - (x == P ? 1.0 : 0.0)) * a;
-    if (sizeof(T) == 4) reinterpret_cast<float2*>(w.Lrow[sp])[(size_t)x * KS_MAX + p] = df_split(val);
-    else w.Lrow[sp][(size_t)x * KS_MAX + p] = val;
-  }
-      });
-}
+// Lp = L Binv with L[x, p] = (G_ext[x, P_p] - delta) a_p, UL_R rows an item, L
+// in shared memory; Rr[p, j] = N_ext[P_p, j] for j < n, stored in the arithmetic
+// type A of the update product.  Per thread: one output (FP64 path) or four
+// consecutive outputs of a row (mixed path: four independent double-float chains
+// sharing the loads of L).  FP64-grade on both paths (B^-1 carries the
+// conditioning of the window): FP64, or double-float on FP32 pairs on the mixed
+// path.  (L by a kernel of its own cost a launch, 4 us of the about 100 us of a
+// small window.)
+constexpr int UL_R = 8;
 
-// Lp = Lrow Binv on the same rows ; Rr[p, j] = N_ext[P_p, j] for j < n,
-// stored in the arithmetic type A of the update product
-// Per thread: one output (FP64 path) or four consecutive outputs of a row
-// (mixed path: four independent double-float chains sharing the loads of L).
 template <typename T, typename A>
 __global__ void __launch_bounds__(256) k_upd_lp_rr(Config cfg) {
   constexpr int PT = sizeof(T) == 4 ? 4 : 1;
+  using S = typename std::conditional<sizeof(T) == 4, float2, double>::type;
+  __shared__ S s_L[UL_R][KS_MAX + 1];
   for_each_item(
       2 * cfg.n_walkers,
       [&](int s) -> long long {
         const WalkerDev& w = cfg.W[s >> 1];
         if (!upd_active(w)) return 0;
-        const int lq = (w.n_acc + PT - 1) / PT;
-        return blocks_of((long long)(w.n + w.n_ins) * lq, 256) + blocks_of((long long)w.n_acc * w.n, 256);
+        return blocks_of(w.n + w.n_ins, UL_R) + blocks_of((long long)w.n_acc * w.n, 256);
       },
       [&](int s, int item) {
         const WalkerDev& w = cfg.W[s >> 1];
+        const ProblemDev& pb = cfg.P[w.problem];
         const int sp = s & 1;
         const int l = w.n_acc, n = w.n, rows = n + w.n_ins;
-        const int lq = (l + PT - 1) / PT;
-        const int lp_blocks = (int)blocks_of((long long)rows * lq, 256);
+        const int lp_blocks = (int)blocks_of(rows, UL_R);
+        const ExtView<T> v = make_view<T>(w, sp);
         if (item < lp_blocks) {
-          const int idx = item * 256 + threadIdx.x;
-          if (idx < rows * lq) {
-            const int t = idx / lq, p = (idx - t * lq) * PT;
-            const int x = upd_row(w, t);
-            // FP64-grade on both paths (B^-1 carries the conditioning of the
-            // window): FP64, or double-float on FP32 pairs on the mixed path
-            if (sizeof(T) == 4) {
-              const float2* Lr = reinterpret_cast<const float2*>(w.Lrow[sp]) + (size_t)x * KS_MAX;
+          const int t0 = item * UL_R, nr = min(UL_R, rows - t0);
+          __syncthreads();  // the previous item is done with the rows of L
+          for (int e = threadIdx.x; e < nr * l; e += 256) {
+            const int r = e / l, p = e - r * l;
+            const int x = upd_row(w, t0 + r), P = w.P[p];
+            const double a = w.aP[sp][p];
+            double val = 0.0;
+            if (a != 0.0 && !(x < n && v.vs[x] == 0)) val = (g_ext(v, pb, sp, x, P) - (x == P ? 1.0 : 0.0)) * a;
+            if constexpr (sizeof(T) == 4) s_L[r][p] = df_split(val);
+            else s_L[r][p] = val;
+          }
+          __syncthreads();
+          const int lq = (l + PT - 1) / PT;
+          for (int e = threadIdx.x; e < nr * lq; e += 256) {
+            const int r = e / lq, p = (e - r * lq) * PT;
+            const int x = upd_row(w, t0 + r);
+            if constexpr (sizeof(T) == 4) {
               const float2* Bi = reinterpret_cast<const float2*>(w.Binv[sp]);
               float hi[PT], lo[PT];
 #pragma unroll
               for (int u = 0; u < PT; ++u) hi[u] = lo[u] = 0.f;
               for (int q = 0; q < l; ++q) {
-                const float2 a = Lr[q];
+                const float2 a = s_L[r][q];
                 const float2* brow = Bi + (size_t)q * KS_MAX + p;
 #pragma unroll
                 for (int u = 0; u < PT; ++u) {
@@ -992,17 +980,15 @@ __global__ void __launch_bounds__(256) k_upd_lp_rr(Config cfg) {
               for (int u = 0; u < PT; ++u)
                 if (p + u < l) out[u] = df_norm(hi[u], lo[u]);
             } else {
-              const double* Lr = w.Lrow[sp] + (size_t)x * KS_MAX;
               const double* Bi = w.Binv[sp];
               double acc = 0.0;
-              for (int q = 0; q < l; ++q) acc += Lr[q] * Bi[(size_t)q * KS_MAX + p];
+              for (int q = 0; q < l; ++q) acc += s_L[r][q] * Bi[(size_t)q * KS_MAX + p];
               w.Lp[sp][(size_t)x * KS_MAX + p] = acc;
             }
           }
         } else {
           const int idx = (item - lp_blocks) * 256 + threadIdx.x;
           if (idx < l * n) {
-            const ExtView<T> v = make_view<T>(w, sp);
             const int p = idx / n, j = idx - p * n;
             const int P = w.P[p];
             ((A*)w.Rr[sp])[(size_t)p * w.cap + j] =
@@ -1012,10 +998,18 @@ __global__ void __launch_bounds__(256) k_upd_lp_rr(Config cfg) {
       });
 }
 
-// In place: N[i, j] += sum_p Lp[i, p] Rr[p, j] for i, j < n.
-// grid = (col tiles, row tiles, walkers*2), block 256, 32x32 tile.
+// Items of 256 entries of the rows and columns of a window's accepted insertions.
+__device__ __forceinline__ long long border_items(const WalkerDev& w) {
+  if (!upd_active(w) || w.n_ins == 0) return 0;
+  return blocks_of(2LL * w.n_ins * w.n + (long long)w.n_ins * w.n_ins, 256);
+}
+
+// In place: N[i, j] += sum_p Lp[i, p] Rr[p, j] for i, j < n, 32x32 tiles; then
+// the items of the accepted insertions (disjoint entries of N, the same inputs).
 template <typename T, typename A>
 __device__ __forceinline__ void upd_apply_tile(const Config& cfg, int wi, int sp, int tile);
+template <typename T, typename A>
+__device__ __forceinline__ void upd_border_item(const Config& cfg, int wi, int sp, int item);
 
 template <typename T, typename A>
 __global__ void __launch_bounds__(256) k_upd_apply(Config cfg) {
@@ -1024,9 +1018,13 @@ __global__ void __launch_bounds__(256) k_upd_apply(Config cfg) {
       [&](int s) -> long long {
         const WalkerDev& w = cfg.W[s >> 1];
         const long long t = (w.n + TT - 1) / TT;
-        return upd_active(w) ? t * t : 0;
+        return upd_active(w) ? t * t + border_items(w) : 0;
       },
-      [&](int s, int item) { upd_apply_tile<T, A>(cfg, s >> 1, s & 1, item); });
+      [&](int s, int item) {
+        const int t = (cfg.W[s >> 1].n + TT - 1) / TT;
+        if (item < t * t) upd_apply_tile<T, A>(cfg, s >> 1, s & 1, item);
+        else upd_border_item<T, A>(cfg, s >> 1, s & 1, item - t * t);
+      });
 }
 
 template <typename T, typename A>
@@ -1080,15 +1078,13 @@ __device__ __forceinline__ void upd_apply_tile(const Config& cfg, int wi, int sp
 template <typename T, typename A>
 __global__ void __launch_bounds__(256) k_upd_border(Config cfg) {
   for_each_item(
-      2 * cfg.n_walkers,
-      [&](int s) -> long long {
-        const WalkerDev& w = cfg.W[s >> 1];
-        if (!upd_active(w) || w.n_ins == 0) return 0;
-        return blocks_of(2LL * w.n_ins * w.n + (long long)w.n_ins * w.n_ins, 256);
-      },
-      [&](int s, int item) {
-  const WalkerDev& w = cfg.W[s >> 1];
-  const int sp = s & 1;
+      2 * cfg.n_walkers, [&](int s) -> long long { return border_items(cfg.W[s >> 1]); },
+      [&](int s, int item) { upd_border_item<T, A>(cfg, s >> 1, s & 1, item); });
+}
+
+template <typename T, typename A>
+__device__ __forceinline__ void upd_border_item(const Config& cfg, int wi, int sp, int item) {
+  const WalkerDev& w = cfg.W[wi];
   const int n = w.n, l = w.n_acc, ni = w.n_ins, ld = w.cap;
   T* N = (T*)w.N[w.parity][sp];
   const A* Rr = (const A*)w.Rr[sp];
@@ -1136,7 +1132,6 @@ __global__ void __launch_bounds__(256) k_upd_border(Config cfg) {
       stN(N, (size_t)(n + m) * ld + n + m2, v);
     }
   }
-      });
 }
 
 // Vertex list after the window: removed vertices dead, insertions appended,
@@ -1433,21 +1428,23 @@ static int launch_group_t(int group, const Config& cfg, int max_cap, cudaStream_
         launch_upd_factors(cfg, max_cap, st);
         return 1;
       }
-      k_upd_lrow<T><<<persist_grid((const void*)k_upd_lrow<T>, S * kc, 256), 256, 0, st>>>(cfg);
       k_upd_lp_rr<T, A><<<persist_grid((const void*)k_upd_lp_rr<T, A>, 2 * S * kc, 256), 256, 0, st>>>(cfg);
-      return 2;
+      return 1;
     case GROUP_UPDATE:
       if (cfg.prec == PREC_MIXED && cfg.upd_kernel == UPD_TCGEN05)
         launch_upd_tc(cfg, st);
       else
-        k_upd_apply<T, A><<<grid_for(S * t32 * t32), 256, 0, st>>>(cfg);
+        k_upd_apply<T, A><<<grid_for(S * (t32 * t32 + 2 * kc)), 256, 0, st>>>(cfg);
       return 1;
     case GROUP_UPDATE_POST:
-      k_upd_border<T, A><<<persist_grid((const void*)k_upd_border<T, A>, 2 * S * kc, 256), 256, 0, st>>>(cfg);
+      // (the CUDA-core update has done the insertions' rows and columns)
+      if (sizeof(T) == 4 && cfg.upd_kernel == UPD_TCGEN05)
+        k_upd_border<float, float><<<persist_grid((const void*)k_upd_border<float, float>, 2 * S * kc, 256), 256, 0,
+                                     st>>>(cfg);
       k_window_end<<<W, 256, 0, st>>>(cfg);
       k_compact_N<T><<<persist_grid((const void*)k_compact_N<T>, S * t32 * t32, 256), 256, 0, st>>>(cfg);
       k_compact_end<<<W, 256, 0, st>>>(cfg);
-      return 4;
+      return sizeof(T) == 4 && cfg.upd_kernel == UPD_TCGEN05 ? 4 : 3;
     default:
       return 0;
   }
