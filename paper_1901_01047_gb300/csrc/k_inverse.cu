@@ -389,7 +389,8 @@ __global__ void __launch_bounds__(GJ_THREADS) k_gj_cluster(Config cfg, int mode,
 // by all SMs.  With the update on the cluster's 16 SMs as well, n^3 multiply-adds
 // on 32 a cycle took half the time: dca_fresh_N of order 500 4.33 -> 3.21 ms.  At
 // order 256 the two launches a panel still cost what the update saves (1.59 ms
-// against 1.52 on the cluster), hence GW_MIN.
+// against 1.52 on the cluster), hence GW_MIN.  The panel stays on 16 blocks: with 8
+// a call of order 500 takes 3.41 ms, with 4 3.72.
 constexpr int GW_B = 16, GW_R = 8, GW_C = 64;  // panel; rows and columns of an update item
 constexpr int GW_MIN = 320, GW_MAX = 4096;     // orders that take this path
 
