@@ -9,11 +9,15 @@
 // times powers of two sharing one exponent per row (column),
 //     A[i, k]  = 2^ea_i  sum_s  a_s[i, k] 2^(-9 (s + 1)),   s < 5,
 //     N0[k, j] = 2^eb_j  sum_t  b_t[k, j] 2^(-9 (t + 1)),   t < 4,
-// |a_s|, |b_t| <= 256, each exact in FP16.  A product of two digit planes is
+// |a_s|, |b_t| <= 256, each exact in FP16; the last b_t is not rounded to an
+// integer but to the 11 bits of FP16, so that N0 is cut at 2^-40 of its column
+// maximum and not at 2^-37 (which showed: 16 sites, beta = 16, order 600, G of
+// most chains 2 to 5 times as far from the FP64 walker's as the FP32 rounding of N
+// leaves it; now 0.8 to 1.4 times on 98 chains of 100).  A product of two digit planes is
 // then a matrix of integers: with |a b| <= 2^16, the 128 terms of one chunk
 // of K sum to at most 2^23 for one plane pair and 2^24 for two, so they
 // accumulate without rounding in the FP32 accumulators of tcgen05.mma
-// kind::f16.  The pairs (s, t) with
+// kind::f16 (the last b_t enters none of these exact sums).  The pairs (s, t) with
 // s + t = g share the scale 2^(ea_i + eb_j - 9 (g + 2)) and one accumulator;
 // groups 0 and 1 (the leading 2^-18 and 2^-27 parts) are read out exactly
 // every 128 K and summed in double-float, groups 2 .. 5 (2^-36 and below)
@@ -163,7 +167,7 @@ __global__ void __launch_bounds__(256) k_oz_a(Config cfg) {
 }
 
 // Digit planes of N0, transposed: plane t, row j, column k = digit t of
-// N0[k, j] scaled by 2^-eb_j.  Item = 32 x 32 tile (k0, j0) of N0 over
+// N0[k, j] scaled by 2^-eb_j, the last one with its fraction.  Item = 32 x 32 tile (k0, j0) of N0 over
 // k < kpad, j < n, staged through shared memory for the transposition.
 __global__ void __launch_bounds__(256) k_oz_slice_n(Config cfg) {
   __shared__ __half ts[OZ_SB][32][34];
@@ -190,7 +194,7 @@ __global__ void __launch_bounds__(256) k_oz_slice_n(Config cfg) {
 #pragma unroll
           for (int d = 0; d < OZ_SB; ++d) {
             const float y = x * (float)(1 << OZ_BETA);
-            const float qd = rintf(y);
+            const float qd = d < OZ_SB - 1 ? rintf(y) : y;
             ts[d][c][r] = __float2half_rn(qd);
             x = __fsub_rn(y, qd);  // exact
           }
