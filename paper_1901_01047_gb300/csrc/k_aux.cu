@@ -250,6 +250,7 @@ __global__ void __launch_bounds__(256) k_recompute_adopt(Config cfg) {
     if (rel > w.max_drift) w.max_drift = rel;
     w.drift_bits[0] = 0ull;
     w.drift_bits[1] = 0ull;
+    for (int k = 0; k < 6; ++k) w.newton_bits[k / 3][k % 3] = 0u;
     w.parity = par ^ 1;
     w.n_recomputes++;
     w.rec_flops += 2.0 * 2.0 * (double)n * (double)n * (double)n;
@@ -461,10 +462,10 @@ int launch_recompute(int part, const Config& cfg, int max_cap, int* d_sgn, cudaS
         if (cfg.recompute_oz) {
           launch_refine_oz(cfg, max_cap, st);
           launch_correct_tc(cfg, st);
-          return 4;
+          return 5;
         }
         launch_refine_gemms(cfg, max_cap, st);
-        return 2;
+        return 3;
       }
       launch_gj(cfg, 1, max_cap, d_sgn, st);
       return 1;

@@ -1,6 +1,7 @@
-// k_correct_tc.cu -- correction of the Newton recompute on the 5th generation
-// tensor cores (mixed precision):  N1 = N0 + N0 R,  R = I - A N0 from the
-// digit planes (k_refine_oz, which stores R^T split into two TF32 planes).
+// k_correct_tc.cu -- the terms of the Newton recompute N1 = N0 + N0 R (+ N0 R^2)
+// on the 5th generation tensor cores (mixed precision):  D = N0 R,  R = I - A N0
+// from the digit planes (k_refine_oz, which stores R^T split into two TF32
+// planes), and where newton_second() asks for it D R.
 // 3xTF32 as in the other products with N: hi = tf32(x), lo = tf32(x - hi), and
 // hi hi + hi lo + lo hi accumulate in FP32 in tensor memory; R is of the size
 // of the drift, so the ~2^-22 of |N0| |R| that this leaves is far below the
@@ -14,12 +15,12 @@
 // for storing R transposed and split.  Work item = one such tile of one
 // walker-spin; the CTA (one per SM, 320 threads) streams the inner index 32 at
 // a time through a three-stage ring:
-//   warp 4 (TMA producer)   N0 box (128 rows x 32 columns), R^T hi and lo boxes;
-//   warps 0-3 (converters)  split the N0 box in place into hi and a lo plane,
+//   warp 4 (TMA producer)   N0 (or D) box (128 rows x 32 columns), R^T hi and lo boxes;
+//   warps 0-3 (converters)  split that box in place into hi and a lo plane,
 //                           zeros outside the live rows and columns;
 //   warp 5 (MMA issuer)     4 K steps x 3 tcgen05.mma kind::tf32 (M = N = 128)
 //                           into one of two TMEM accumulators;
-//   warps 6-9 (epilogue)    N1 = N0 + accumulator, while the next tile runs.
+//   warps 6-9 (epilogue)    store the accumulator, while the next tile runs.
 // Every wait is bounded; a timeout sets the walker's status to
 // ST_ERR_TIMEOUT, lets the copies in flight land, frees the tensor memory and
 // returns.
@@ -35,7 +36,7 @@ namespace dca {
 
 namespace {
 
-constexpr int CB = 128;  // tile of N1
+constexpr int CB = 128;  // tile of the product
 
 struct CoLayout {
   static constexpr int BOX = CB * 128;     // 128 rows x 32 FP32 columns
@@ -47,18 +48,20 @@ struct CoLayout {
   static_assert(SMEM + sizeof(ItemPlan) + 1024 <= 232448, "shared memory (dynamic + the static item plan)");
 };
 
+template <bool SECOND>
 __device__ __forceinline__ long long co_items(const Config& cfg, int s) {
   const WalkerDev& w = cfg.W[s >> 1];
   const long long t = (w.n + CB - 1) / CB;
-  return (w.active && w.recompute_pending && w.status == ST_OK) ? t * t : 0;
+  return (w.active && w.recompute_pending && w.status == ST_OK && (!SECOND || newton_second(w, s & 1))) ? t * t : 0;
 }
 
+template <bool SECOND>
 struct CoIter {
   PlanWalk<ItemPlan> pw;
   __device__ void start(const ItemPlan& plan) { pw.start(plan); }
   __device__ bool next(const Config& cfg, int& set, int& i0, int& j0) {
     int sub = 0;
-    if (!pw.next(2 * cfg.n_walkers, [&](int s) { return co_items(cfg, s); }, set, sub)) return false;
+    if (!pw.next(2 * cfg.n_walkers, [&](int s) { return co_items<SECOND>(cfg, s); }, set, sub)) return false;
     const int t = (cfg.W[set >> 1].n + CB - 1) / CB;
     i0 = (sub / t) * CB;
     j0 = (sub % t) * CB;
@@ -68,6 +71,7 @@ struct CoIter {
 
 }  // namespace
 
+template <bool SECOND>
 __global__ void __launch_bounds__(320, 1) k_correct_tc(Config cfg) {
   using L = CoLayout;
   constexpr int S = L::STAGES;
@@ -111,9 +115,9 @@ __global__ void __launch_bounds__(320, 1) k_correct_tc(Config cfg) {
   tc::fence_after_sync();
   const uint32_t tmem = *tmem_slot;
   __shared__ ItemPlan plan;
-  plan_items(plan, 2 * cfg.n_walkers, [&](int s) { return co_items(cfg, s); });
+  plan_items(plan, 2 * cfg.n_walkers, [&](int s) { return co_items<SECOND>(cfg, s); });
 
-  CoIter it;
+  CoIter<SECOND> it;
   it.start(plan);
   int set = 0, i0 = 0, j0 = 0;
   if (warp == 4) {
@@ -127,7 +131,7 @@ __global__ void __launch_bounds__(320, 1) k_correct_tc(Config cfg) {
         const int n = w.n;
         const TmapDev* m = cfg.tmaps + (size_t)set * TMAPS_PER_SPIN;
         const void* mN = m + 2 + w.parity;
-        const void* mN32 = m + 6 + w.parity;        // 32-row boxes: the last, partial row block
+        const void* mN32 = SECOND ? m + 11 : m + 6 + w.parity;  // 32-row boxes: the last, partial row block
         const void* mRh = m + 2 + (w.parity ^ 1);   // R^T hi in the other buffer of N
         const void* mRl = m + 10;                   // R^T lo in the upper half of the FP64 work matrix
         const int nsub = n - i0 >= CB ? 4 : (n - i0 + 31) / 32;  // 32-row boxes that start below n
@@ -141,7 +145,7 @@ __global__ void __launch_bounds__(320, 1) k_correct_tc(Config cfg) {
           const uint32_t s0 = sb + st * L::STAGE;
           tc::mbar_expect_tx(full(st), (uint32_t)(nsub * (L::BOX / 4) + 2 * L::BOX));
           armed[st] = u + 1;
-          if (nsub == 4) {
+          if (!SECOND && nsub == 4) {
             tc::tma_load_2d(s0, mN, k0, i0, full(st));
           } else {
             for (int q = 0; q < nsub; ++q) tc::tma_load_2d(s0 + q * (L::BOX / 4), mN32, k0, i0 + 32 * q, full(st));
@@ -249,10 +253,10 @@ __global__ void __launch_bounds__(320, 1) k_correct_tc(Config cfg) {
     bool stop = false;
     const int sub = warp & 3, r = 32 * sub + lane;
     while (!stop && it.next(cfg, set, i0, j0)) {
-      const WalkerDev& w = cfg.W[set >> 1];
+      WalkerDev& w = cfg.W[set >> 1];
       const int sp = set & 1, n = w.n, ld = w.cap, b = (int)(k & 1u), i = i0 + r;
-      const float* N0 = (const float*)w.N[w.parity][sp];
-      float* N1 = (float*)w.Ascr[sp];
+      float* out = SECOND ? (float*)w.OzN[sp] : (float*)w.Ascr[sp];
+      uint32_t dmax = 0u;
       const bool mine = tc::mbar_wait(afull(b), (k >> 1) & 1u, abort_flag, cfg.wait_cycles);
       if (!__all_sync(0xffffffffu, mine)) {
         stop = true;
@@ -269,22 +273,21 @@ __global__ void __launch_bounds__(320, 1) k_correct_tc(Config cfg) {
           for (int q = 0; q < 8; ++q) {
             const int j = j0 + cb + 4 * q;
             if (j + 3 < n) {
-              float4 x = *reinterpret_cast<const float4*>(N0 + o + 4 * q);
-              x.x += v[4 * q];
-              x.y += v[4 * q + 1];
-              x.z += v[4 * q + 2];
-              x.w += v[4 * q + 3];
-              *reinterpret_cast<float4*>(N1 + o + 4 * q) = x;
+              *reinterpret_cast<float4*>(out + o + 4 * q) =
+                  make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
             } else {
 #pragma unroll
               for (int e = 0; e < 4; ++e)
-                if (j + e < n) N1[o + 4 * q + e] = N0[o + 4 * q + e] + v[4 * q + e];
+                if (j + e < n) out[o + 4 * q + e] = v[4 * q + e];
             }
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+              if (j + e < n) dmax = max(dmax, abs_bits(v[4 * q + e]));
           }
         }
       }
       tc::fence_before_sync();
-      __syncwarp();
+      newton_max(&w.newton_bits[sp][SECOND ? 2 : 1], dmax);  // converges the warp
       if (lane == 0) tc::mbar_arrive(aempty(b));
       ++k;
     }
@@ -305,11 +308,15 @@ __global__ void __launch_bounds__(320, 1) k_correct_tc(Config cfg) {
 }
 
 cudaError_t setup_correct_tc() {
-  return cudaFuncSetAttribute(k_correct_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, CoLayout::SMEM);
+  const cudaError_t e =
+      cudaFuncSetAttribute(k_correct_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, CoLayout::SMEM);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_correct_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, CoLayout::SMEM);
 }
 
 void launch_correct_tc(const Config& cfg, cudaStream_t st) {
-  k_correct_tc<<<device_sm_count(), 320, CoLayout::SMEM, st>>>(cfg);
+  k_correct_tc<false><<<device_sm_count(), 320, CoLayout::SMEM, st>>>(cfg);
+  k_correct_tc<true><<<device_sm_count(), 320, CoLayout::SMEM, st>>>(cfg);
 }
 
 }  // namespace dca

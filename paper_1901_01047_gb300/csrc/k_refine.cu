@@ -5,8 +5,15 @@
 //     R  = I - A N0      FP64-grade (double-float products and sums)
 //     N1 = N0 + N0 R     FP32 (R is of the size of the drift; with the residual
 //                        from digit planes 3xTF32, k_correct_tc.cu)
-// One step squares the relative error of N0: an FP32 N0 that drifted by 1e-5
-// comes back to the FP32 rounding level.  Both products are tiled GEMMs on a
+// One step leaves N0 R^2: an FP32 N0 that drifted by 1e-5 comes back to the
+// FP32 rounding level.  After a window close to singular R can be far larger,
+// and rows of N enter G with e^V - 1 (1.5e3 at 16 sites, beta = 16): on one of 100
+// chains there (order 590, max |R| = 0.03, condition number 4e8) one step left
+// 1.5e-4 of G, another build 2.7e-3.  So where max |R| of a walker-spin is 1e-4 or
+// more, the next term of N1 = N0 (I + R + R^2 + ...) follows, (N0 R) R from the
+// first one, by the same kernel; it is added if it is no more than half the first.
+// That chain's G: 1.4e-5, with the Gauss-Jordan inverse 7e-6.  The launch costs a
+// pass 1 to 2 %, also where no walker needs it.  Both products are tiled GEMMs on a
 // persistent grid over (walker-spin, 64 x 64 output tile), so one walker's
 // recompute spreads over every SM.  The residual is the whole cost; it runs
 // on the FP32 pipes in double-float arithmetic because GB300's FP64 units
@@ -14,9 +21,10 @@
 //
 // Buffers (the recompute follows a compaction, all n rows live):
 //   A   Ascr[sp] (FP32 pairs)    -> R  into N[parity ^ 1][sp] (FP32; from the digit planes R^T, see k_refine_tc.cu)
-//   N0  N[parity][sp]            -> N1 into Ascr[sp] viewed as FP32
-// k_refine_adopt then measures the drift max|N1 - N0| / max|N1| and copies
-// N1 into N[parity ^ 1][sp] for the parity switch.
+//   N0  N[parity][sp]            -> N0 R into Ascr[sp] viewed as FP32
+//   N0 R                         -> N0 R^2 into the upper half of Ascr[sp] (digit planes: into OzN, no longer needed)
+// k_refine_adopt then forms N1 in N[parity ^ 1][sp] for the parity switch, with
+// the drift max|N1 - N0| / max|N1|.
 #include <cstdint>
 
 #include "device_util.cuh"
@@ -62,6 +70,7 @@ __global__ void __launch_bounds__(256) k_refine_resid(Config cfg) {
         float* R = (float*)w.N[w.parity ^ 1][sp];
         const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
         float hi[4][4], lo[4][4];
+        uint32_t rmax = 0u;
 #pragma unroll
         for (int a = 0; a < 4; ++a)
 #pragma unroll
@@ -113,21 +122,25 @@ __global__ void __launch_bounds__(256) k_refine_resid(Config cfg) {
             if (i < n && j < n) {
               // (delta - hi) - lo, the difference of nearly equal numbers taken exactly first
               const float d = __fsub_rn(i == j ? 1.0f : 0.0f, hi[a][b]);
-              R[(size_t)i * ld + j] = __fsub_rn(d, lo[a][b]);
+              const float v = __fsub_rn(d, lo[a][b]);
+              R[(size_t)i * ld + j] = v;
+              rmax = max(rmax, abs_bits(v));
             }
           }
         }
+        newton_max(&cfg.W[s >> 1].newton_bits[sp][0], rmax);
       });
 }
 
-// N1 = N0 + N0 R, FP32, into Ascr[sp] viewed as FP32 (ld = cap).  Item =
-// 128 x 128 output tile; thread (tx, ty) of 16 x 16 owns rows ty 4 + a +
+// N0 R, FP32, into Ascr[sp] viewed as FP32 (ld = cap); SECOND: (N0 R) R into its
+// upper half, for the walker-spins that need it.  Item = 128 x 128 output tile; thread (tx, ty) of 16 x 16 owns rows ty 4 + a +
 // 64 p and columns tx 4 + b + 64 q (a, b < 4; p, q < 2): 64 accumulators and
 // four 16-byte shared-memory reads per 64 FMAs.  The next K step's tiles are
 // loaded into registers while the current one is multiplied.
 constexpr int CT = 128;  // output tile
 constexpr int CK = 16;   // K step
 
+template <bool SECOND>
 __global__ void __launch_bounds__(256) k_refine_correct(Config cfg) {
   __shared__ __align__(16) float As[CK][CT + 4];  // [k][i] of N0
   __shared__ __align__(16) float Bs[CK][CT + 4];  // [k][j] of R
@@ -136,16 +149,17 @@ __global__ void __launch_bounds__(256) k_refine_correct(Config cfg) {
       [&](int s) -> long long {
         const WalkerDev& w = cfg.W[s >> 1];
         const long long t = (w.n + CT - 1) / CT;
-        return refine_wants(w) ? t * t : 0;
+        return refine_wants(w) && (!SECOND || newton_second(w, s & 1)) ? t * t : 0;
       },
       [&](int s, int item) {
         const WalkerDev& w = cfg.W[s >> 1];
         const int sp = s & 1, n = w.n, ld = w.cap;
         const int tiles = (n + CT - 1) / CT;
         const int i0 = (item / tiles) * CT, j0 = (item - (item / tiles) * tiles) * CT;
-        const float* N0 = (const float*)w.N[w.parity][sp];
+        float* const D = (float*)w.Ascr[sp];
+        const float* N0 = SECOND ? D : (const float*)w.N[w.parity][sp];
         const float* R = (const float*)w.N[w.parity ^ 1][sp];
-        float* N1 = (float*)w.Ascr[sp];
+        float* out = SECOND ? D + (size_t)ld * ld : D;
         const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
         float ra[8], rb[8];  // the next K step: A rows (k fastest), R rows (j fastest)
         auto fetch = [&](int k0) {
@@ -159,6 +173,7 @@ __global__ void __launch_bounds__(256) k_refine_correct(Config cfg) {
           }
         };
         float acc[8][8];
+        uint32_t dmax = 0u;
 #pragma unroll
         for (int a = 0; a < 8; ++a)
 #pragma unroll
@@ -200,26 +215,27 @@ __global__ void __launch_bounds__(256) k_refine_correct(Config cfg) {
             const int j = j0 + tx * 4 + 64 * q;  // 16-byte aligned: ld and j0 are multiples of 4
             const size_t o = (size_t)i * ld + j;
             if (j + 3 < n) {
-              float4 v = *reinterpret_cast<const float4*>(N0 + o);
-              v.x += acc[a][4 * q];
-              v.y += acc[a][4 * q + 1];
-              v.z += acc[a][4 * q + 2];
-              v.w += acc[a][4 * q + 3];
-              *reinterpret_cast<float4*>(N1 + o) = v;
+              *reinterpret_cast<float4*>(out + o) =
+                  make_float4(acc[a][4 * q], acc[a][4 * q + 1], acc[a][4 * q + 2], acc[a][4 * q + 3]);
             } else {
 #pragma unroll
               for (int b = 0; b < 4; ++b)
-                if (j + b < n) N1[o + b] = N0[o + b] + acc[a][4 * q + b];
+                if (j + b < n) out[o + b] = acc[a][4 * q + b];
             }
+#pragma unroll
+            for (int b = 0; b < 4; ++b)
+              if (j + b < n) dmax = max(dmax, abs_bits(acc[a][4 * q + b]));
           }
         }
+        newton_max(&cfg.W[s >> 1].newton_bits[sp][SECOND ? 2 : 1], dmax);
       });
 }
 
-// Drift max|N1 - N0| and max|N1| (atomicMax on the bits of non-negative
-// doubles, folded into the walker by k_recompute_adopt) and the copy of N1
-// into N[parity ^ 1].  Bound by memory: item = 32 rows x 128 columns, 16-byte
-// accesses, a thread's eight loads in flight together.  The largest difference
+// N1 = N0 + N0 R (+ N0 R^2, both terms added before the one rounding to N1) into
+// N[parity ^ 1], with the drift max|N1 - N0| and max|N1| (atomicMax on the bits of
+// non-negative doubles, folded into the walker by k_recompute_adopt).  Bound by
+// memory: item = 32 rows x 128 columns, 16-byte accesses, a thread's eight loads
+// in flight together.  The largest difference
 // is searched in FP32 (rounding keeps the order) and only its pair subtracted
 // in FP64; with an FP64 difference per entry and an integer division for its
 // row the batch of 256 took 0.71 ms, now 0.12.
@@ -241,7 +257,10 @@ __global__ void __launch_bounds__(256) k_refine_adopt(Config cfg) {
         const int cblocks = (n + AD_C - 1) / AD_C;
         const int i0 = (item / cblocks) * AD_R + warp, j = (item % cblocks) * AD_C + 4 * lane;
         const float* N0 = (const float*)w.N[w.parity][sp];
-        const float* N1 = (const float*)w.Ascr[sp];
+        const float* D = (const float*)w.Ascr[sp];
+        const float* D2 = cfg.recompute_oz ? (const float*)w.OzN[sp] : D + (size_t)ld * ld;
+        const bool second = newton_second(w, sp) && __uint_as_float(w.newton_bits[sp][2]) <=
+                                                        0.5f * __uint_as_float(w.newton_bits[sp][1]);
         float* dst = (float*)w.N[w.parity ^ 1][sp];
         constexpr int U = AD_R / 8;
         float4 a[U], b[U];
@@ -250,8 +269,19 @@ __global__ void __launch_bounds__(256) k_refine_adopt(Config cfg) {
           const bool in = i0 + 8 * u < n && j < n;
           const size_t o = (size_t)(i0 + 8 * u) * ld + j;
           a[u] = in ? *reinterpret_cast<const float4*>(N0 + o) : make_float4(0.f, 0.f, 0.f, 0.f);
-          b[u] = in ? *reinterpret_cast<const float4*>(N1 + o) : make_float4(0.f, 0.f, 0.f, 0.f);
+          b[u] = in ? *reinterpret_cast<const float4*>(D + o) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
+        if (second) {
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            if (i0 + 8 * u >= n || j >= n) continue;
+            const float4 c = *reinterpret_cast<const float4*>(D2 + (size_t)(i0 + 8 * u) * ld + j);
+            b[u] = make_float4(b[u].x + c.x, b[u].y + c.y, b[u].z + c.z, b[u].w + c.w);
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          b[u] = make_float4(a[u].x + b[u].x, a[u].y + b[u].y, a[u].z + b[u].z, a[u].w + b[u].w);
         float dmax = 0.0f, pa = 0.0f, pb = 0.0f, nmax = 0.0f;
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -313,7 +343,8 @@ void launch_refine_gemms(const Config& cfg, int max_cap, cudaStream_t st) {
 void launch_refine_correct(const Config& cfg, int max_cap, cudaStream_t st) {
   const long long t = (max_cap + CT - 1) / CT;
   const long long items = 2LL * cfg.n_walkers * t * t;
-  k_refine_correct<<<persist_grid((const void*)k_refine_correct, items, 256), 256, 0, st>>>(cfg);
+  k_refine_correct<false><<<persist_grid((const void*)k_refine_correct<false>, items, 256), 256, 0, st>>>(cfg);
+  k_refine_correct<true><<<persist_grid((const void*)k_refine_correct<true>, items, 256), 256, 0, st>>>(cfg);
 }
 
 void launch_refine_adopt(const Config& cfg, int max_cap, cudaStream_t st) {

@@ -492,6 +492,7 @@ __global__ void __launch_bounds__(192, 1) k_refine_oz(Config cfg) {
       // two TF32 planes: K-major operands of the correction N0 R (k_correct_tc),
       // with zeros up to the 32-column padding of its last K step
       const int j = j0 + r;
+      uint32_t rmax = 0u;
       if (j < n) {
         const int eb = w.OzE[sp][ld + j], n32 = (n + 31) & ~31;
         float* Rh = (float*)w.N[w.parity ^ 1][sp] + (size_t)j * ld;
@@ -508,6 +509,7 @@ __global__ void __launch_bounds__(192, 1) k_refine_oz(Config cfg) {
               const int e = w.OzE[sp][i] + eb - 2 * OZ_BETA;
               const float d = __fsub_rn(i == j ? 1.0f : 0.0f, ldexpf(h[x + y], e));
               v = __fsub_rn(d, ldexpf(l[x + y], e));
+              rmax = max(rmax, abs_bits(v));
             }
             tc::tf32_split(v, hi[y], lo[y]);
           }
@@ -515,6 +517,7 @@ __global__ void __launch_bounds__(192, 1) k_refine_oz(Config cfg) {
           oz_store8(Rl + i0 + x, lo);
         }
       }
+      newton_max(&cfg.W[set >> 1].newton_bits[sp][0], rmax);
     }
     if (stop && threadIdx.x == 0) set_status(cfg.W[set >> 1], ST_ERR_TIMEOUT);
   }

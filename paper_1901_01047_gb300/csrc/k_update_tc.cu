@@ -662,6 +662,8 @@ bool encode_update_maps(const WalkerDev& w, int ks, int upd_bn, TmapDev* out) {
     if (w.OzA[sp] && !encode_2d_f16(m + 9, w.OzA[sp], C, 5 * C, 64u)) return false;
     // low TF32 plane of R^T in the recompute correction
     if (w.Ascr[sp] && !encode_2d(m + 10, reinterpret_cast<float*>(w.Ascr[sp]) + C * C, C, C, C * 4, TC_BM)) return false;
+    // and its first term N0 R
+    if (w.Ascr[sp] && !encode_2d(m + 11, w.Ascr[sp], C, C, C * 4, 32u)) return false;
   }
   return true;
 }

@@ -63,11 +63,11 @@ size_t gj_wide_scratch(int n);
 bool launch_gj_wide(const Config& cfg, int n, int* d_sgn, cudaStream_t st);
 // Gauss-Jordan inverse of the FP64 work matrices, one 8-block cluster each.
 void launch_gj(const Config& cfg, int mode, int max_n, int* d_sgn, cudaStream_t st);
-// Mixed-precision recompute by one Newton step against the FP64 A = N^-1:
-// the two products (R = I - A N0 in FP64, N1 = N0 + N0 R in FP32), then the
-// drift measurement and the copy of N1 into the other buffer.
+// Mixed-precision recompute by a Newton step against the FP64 A = N^-1: the
+// products (R = I - A N0 in FP64, N0 R in FP32 and where R is large N0 R^2), then
+// N1 = N0 + N0 R (+ N0 R^2) into the other buffer with the drift.
 void launch_refine_gemms(const Config& cfg, int max_cap, cudaStream_t st);
-// N1 = N0 + N0 R: FP32 for the double-float residual's R, 3xTF32 tcgen05 for
+// N0 R and N0 R^2: FP32 for the double-float residual's R, 3xTF32 tcgen05 for
 // the split R^T of the digit planes.
 cudaError_t setup_correct_tc();
 void launch_correct_tc(const Config& cfg, cudaStream_t st);

@@ -113,6 +113,8 @@ struct WalkerDev {
   int64_t n_prop, n_accept, n_ties, n_aborts, n_windows, n_meas, n_recomputes;
   double sign_sum, k_sum, max_drift;
   unsigned long long drift_bits[2];  // max |N_old - N_new| and max |N_new| of a recompute (bits of doubles >= 0)
+  // Newton recompute, per spin: max |R|, |N0 R| and |N0 R^2| (bits of |FP32|, so that a NaN is the largest)
+  uint32_t newton_bits[2][3];
   // algorithmic work (both spins): N update flop / bytes, candidate extension flop / bytes
   double flops, upd_bytes, ext_flops, ext_bytes, rec_flops;
 
@@ -174,6 +176,22 @@ struct WalkerDev {
 // A walker keeps its first error: later kernels of the same window may meet
 // the consequences of the first failure, which would hide its cause.
 __device__ __forceinline__ void set_status(WalkerDev& w, int32_t code) { atomicCAS(&w.status, (int32_t)ST_OK, code); }
+
+// Whether the Newton recompute of a walker-spin takes its second term N0 R^2
+// (k_refine.cu): max |R| from NEWTON_R_MIN on, where what one term leaves reaches
+// the FP32 rounding of N, and below 1, past which the series does not converge
+// (NaN and infinity order above).
+constexpr float NEWTON_R_MIN = 1e-4f;
+__device__ __forceinline__ bool newton_second(const WalkerDev& w, int sp) {
+  return w.newton_bits[sp][0] >= __float_as_uint(NEWTON_R_MIN) && w.newton_bits[sp][0] < __float_as_uint(1.0f);
+}
+
+// Largest of the warp's values (bits of |x|) into *to.
+__device__ __forceinline__ void newton_max(uint32_t* to, uint32_t m) {
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) atomicMax(to, m);
+}
+__device__ __forceinline__ uint32_t abs_bits(float x) { return __float_as_uint(x) & 0x7fffffffu; }
 #endif
 
 // Iteration state of the device-side window loop.  iters and max_iters are
@@ -203,8 +221,9 @@ struct PoolState {
 // and 1 (128-row boxes), the candidate tables V and U of the tensor-core
 // extension, N of parity 0 and 1 in 32-row boxes (MN-major operand), the
 // digit planes of the sliced recompute residual (N: 128-row boxes, A: 64), the
-// low plane of R^T of the recompute correction (upper half of Ascr).
-constexpr int TMAPS_PER_SPIN = 11;
+// low plane of R^T of the recompute correction (upper half of Ascr), its first
+// term N0 R (lower half of Ascr, 32-row boxes).
+constexpr int TMAPS_PER_SPIN = 12;
 
 // Opaque copy of a TMA tensor map (CUtensorMap: 128 bytes, 64-byte aligned).
 struct alignas(64) TmapDev {

@@ -1531,6 +1531,7 @@ extern "C" DCA_API int dca_walker_load(dca_walker* h, const void* buf, size_t n)
     w.k_sum = sw.k_sum;
     w.max_drift = sw.max_drift;
     w.drift_bits[0] = w.drift_bits[1] = 0ull;
+    for (auto& sp : w.newton_bits) sp[0] = sp[1] = sp[2] = 0u;
     w.flops = sw.flops;
     w.upd_bytes = sw.upd_bytes;
     w.ext_flops = sw.ext_flops;
