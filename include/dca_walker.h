@@ -72,13 +72,15 @@ extern "C" {
  *           accumulation; the update factors L B^-1 and the rows of accepted
  *           insertions in double-float (FP32 pairs, about 44 bits); Gamma (B^-1) and
  *           the determinant ratios in FP64 (DCA_GAMMA_FP64) or double-float
- *           (DCA_GAMMA_DOUBLE_FLOAT); the recompute from an FP64 A = N^-1 with a
- *           double-float residual.  The FP32 storage of N bounds the accuracy: the
- *           measured errors of N and G against the FP64 walker on the same trajectory
- *           are 1e-6..1e-4 relative, growing with the conditioning of N^-1 and with
- *           the updates since the last recompute; with N recomputed before every
- *           measurement (recompute_at_measure) the accumulated G is within about
- *           3e-7.
+ *           (DCA_GAMMA_DOUBLE_FLOAT); the recompute from an FP64 A = N^-1 with an
+ *           FP64-grade residual R, the terms N R and N R^2 in 3xTF32 summed to FP32
+ *           accuracy (DCA_RECOMPUTE_AUTO) or in FP32.  The FP32 storage of N bounds
+ *           the accuracy: the measured errors of N and G against the FP64 walker on
+ *           the same trajectory are 1e-6..1e-4 relative, growing with the conditioning
+ *           of N^-1 and with the updates since the last recompute; with N recomputed
+ *           before every measurement (recompute_at_measure) the accumulated G is within
+ *           about 3e-7 (condition numbers up to 1e5), 0.3e-6 to 1.4e-5 at 16 sites and
+ *           beta = 16 (1e6 to 4e8), as with N from the Gauss-Jordan inverse.
  *   TF32:   as MIXED with one TF32 product per K step instead of three (the
  *           tensor-core kernels only); about 11 bits per product. */
 #define DCA_PREC_FP64 0

@@ -2,25 +2,33 @@
 // on the 5th generation tensor cores (mixed precision):  D = N0 R,  R = I - A N0
 // from the digit planes (k_refine_oz, which stores R^T split into two TF32
 // planes), and where newton_second() asks for it D R.
-// 3xTF32 as in the other products with N: hi = tf32(x), lo = tf32(x - hi), and
-// hi hi + hi lo + lo hi accumulate in FP32 in tensor memory; R is of the size
-// of the drift, so the ~2^-22 of |N0| |R| that this leaves is far below the
-// FP32 rounding of N1.
+// 3xTF32 as in the other products with N: hi = tf32(x), lo = tf32(x - hi) and
+// hi hi + hi lo + lo hi.  The tensor cores truncate when they add to an accumulator,
+// so the hi hi products of every 32 inner indexes go to an accumulator of their
+// own, added in FP32 registers; the cross terms, 2^-12 of them, have one for the
+// whole item.  Error of N0 R against 64 bits, relative, random matrices of order
+// 40 / 129 / 300 / 900: 1.2e-7 / 1.4e-7 / 1.4e-7 / 1.7e-7, the FP32 kernel
+// (k_refine_correct) 1.1e-7 / 2.1e-7 / 3.1e-7 / 5.4e-7, one accumulator for all
+// 3.4e-7 / 1.0e-6 / 2.2e-6 / 6.4e-6 (below order 40 up to twice the FP32 kernel's,
+// of a term that is then below the rounding of N1).  Time of one walker of order
+// 670 / 900: 35.1 / 43.2 us with the second term's idle launch, with one
+// accumulator 34.6 / 39.4, the FP32 kernel 94 / 117.
 //
 // Bound: 3 x 2 n^3 flop per spin at the TF32 rate (the FP32 pipes, where
 // k_refine_correct runs at their peak, are 12 times slower); every 128 x 128
 // tile of N1 re-reads 2 x 128 rows from L2.  256 walkers of orders 90 to 900:
 // 1.84 -> 0.46 ms a recompute, and a pass of the batch 15.4 -> 13.9 ms; 4
-// walkers of 36 sites 9.47 -> 8.95 ms.  The residual kernel pays 0.3 ms of it
-// for storing R transposed and split.  Work item = one such tile of one
-// walker-spin; the CTA (one per SM, 320 threads) streams the inner index 32 at
-// a time through a three-stage ring:
+// walkers of 36 sites 9.47 -> 8.95 ms (both with one accumulator).  The residual
+// kernel pays 0.3 ms of it for storing R transposed and split.  Work item = one
+// such tile of one walker-spin; the CTA (one per SM, 448 threads) streams the
+// inner index 32 at a time through a three-stage ring:
 //   warp 4 (TMA producer)   N0 (or D) box (128 rows x 32 columns), R^T hi and lo boxes;
 //   warps 0-3 (converters)  split that box in place into hi and a lo plane,
 //                           zeros outside the live rows and columns;
-//   warp 5 (MMA issuer)     4 K steps x 3 tcgen05.mma kind::tf32 (M = N = 128)
-//                           into one of two TMEM accumulators;
-//   warps 6-9 (epilogue)    store the accumulator, while the next tile runs.
+//   warp 5 (MMA issuer)     4 K steps x 3 tcgen05.mma kind::tf32 (M = N = 128):
+//                           hi hi into one of two TMEM accumulators in turn,
+//                           the cross terms into one of two others per item;
+//   warps 6-13 (epilogue)   add the chunks up, store the sum at the item's end.
 // Every wait is bounded; a timeout sets the walker's status to
 // ST_ERR_TIMEOUT, lets the copies in flight land, frees the tensor memory and
 // returns.
@@ -36,7 +44,9 @@ namespace dca {
 
 namespace {
 
-constexpr int CB = 128;  // tile of the product
+constexpr int CB = 128;        // tile of the product
+constexpr int CE = 64;         // its columns per epilogue warp
+constexpr int CO_THREADS = 448;  // converters 0-3, producer 4, issuer 5, epilogue 6-13
 
 struct CoLayout {
   static constexpr int BOX = CB * 128;     // 128 rows x 32 FP32 columns
@@ -44,7 +54,7 @@ struct CoLayout {
   static constexpr int STAGES = 3;
   static constexpr int OFF_BAR = STAGES * STAGE;
   static constexpr int SMEM = OFF_BAR + 256 + 1024;
-  static constexpr uint32_t TMEM_COLS = 2 * CB;
+  static constexpr uint32_t TMEM_COLS = 4 * CB;
   static_assert(SMEM + sizeof(ItemPlan) + 1024 <= 232448, "shared memory (dynamic + the static item plan)");
 };
 
@@ -72,7 +82,7 @@ struct CoIter {
 }  // namespace
 
 template <bool SECOND>
-__global__ void __launch_bounds__(320, 1) k_correct_tc(Config cfg) {
+__global__ void __launch_bounds__(CO_THREADS, 1) k_correct_tc(Config cfg) {
   using L = CoLayout;
   constexpr int S = L::STAGES;
   extern __shared__ uint8_t co_raw[];
@@ -100,7 +110,7 @@ __global__ void __launch_bounds__(320, 1) k_correct_tc(Config cfg) {
     }
     for (int b = 0; b < 2; ++b) {
       tc::mbar_init(afull(b), 1);
-      tc::mbar_init(aempty(b), 4);
+      tc::mbar_init(aempty(b), 8);
     }
     tc::mbar_init(fin, 1);
     *abort_flag = 0;
@@ -164,42 +174,39 @@ __global__ void __launch_bounds__(320, 1) k_correct_tc(Config cfg) {
   } else if (warp == 5) {
     // ---------------- MMA issuer ----------------
     if (lane == 0) {
-      uint32_t g = 0, k = 0;
+      uint32_t g = 0, k = 0;  // chunks and items so far
       bool ok = true;
       constexpr uint32_t idesc = tc::idesc_tf32(CB, CB);
       while (ok && it.next(cfg, set, i0, j0)) {
         const int n = cfg.W[set >> 1].n;
-        const int b = (int)(k & 1u);
-        if (k >= 2 && !tc::mbar_wait(aempty(b), ((k >> 1) - 1) & 1u, abort_flag, cfg.wait_cycles)) {
-          ok = false;
-          break;
-        }
-        tc::fence_after_sync();
-        const uint32_t d = tmem + (uint32_t)(CB * b);
-        bool first = true;
+        // read out two items ago, before that item's last chunk was released
+        const uint32_t x = tmem + (uint32_t)(2 * CB + CB * (int)(k & 1u));
         for (int k0 = 0; k0 < n; k0 += 32, ++g) {
-          const int st = (int)(g % S);
+          const int st = (int)(g % S), b = (int)(g & 1u);
           const uint32_t u = g / S;
+          if (g >= 2 && !tc::mbar_wait(aempty(b), ((g >> 1) - 1) & 1u, abort_flag, cfg.wait_cycles)) {
+            ok = false;
+            break;
+          }
           if (!tc::mbar_wait(conv(st), u & 1u, abort_flag, cfg.wait_cycles)) {
             ok = false;
             break;
           }
           tc::fence_after_sync();
+          const uint32_t d = tmem + (uint32_t)(CB * b);
           const uint32_t s0 = sb + st * L::STAGE;
 #pragma unroll
           for (int q = 0; q < 4; ++q) {  // K step of 8 columns: 32 bytes inside the 128-byte swizzle row
             const uint64_t ah = tc::sdesc_k_sw128(s0 + 32 * q), al = tc::sdesc_k_sw128(s0 + L::BOX + 32 * q);
             const uint64_t bh = tc::sdesc_k_sw128(s0 + 2 * L::BOX + 32 * q);
             const uint64_t bl = tc::sdesc_k_sw128(s0 + 3 * L::BOX + 32 * q);
-            tc::mma_tf32(d, ah, bh, idesc, first ? 0u : 1u);
-            tc::mma_tf32(d, ah, bl, idesc, 1u);
-            tc::mma_tf32(d, al, bh, idesc, 1u);
-            first = false;
+            tc::mma_tf32(d, ah, bh, idesc, q > 0 ? 1u : 0u);
+            tc::mma_tf32(x, ah, bl, idesc, k0 + q > 0 ? 1u : 0u);
+            tc::mma_tf32(x, al, bh, idesc, 1u);
           }
           tc::mma_commit(empty(st));
+          tc::mma_commit(afull(b));  // the chunk (and, at the item's end, the cross terms)
         }
-        if (!ok) break;
-        tc::mma_commit(afull(b));
         ++k;
       }
       if (!ok) set_status(cfg.W[set >> 1], ST_ERR_TIMEOUT);
@@ -248,48 +255,68 @@ __global__ void __launch_bounds__(320, 1) k_correct_tc(Config cfg) {
     if (stop && lane == 0) set_status(cfg.W[set >> 1], ST_ERR_TIMEOUT);
     if (stop) *abort_flag = 1;
   } else {
-    // ---------------- epilogue: warps 6-9, TMEM lanes 32 (warp % 4) .. +31 ----------------
-    uint32_t k = 0;
+    // ---------------- epilogue: warps 6-13, TMEM lanes 32 (warp % 4) .. +31, CE columns ----------------
+    uint32_t g = 0, k = 0;  // chunks and items so far
     bool stop = false;
-    const int sub = warp & 3, r = 32 * sub + lane;
+    const int sub = warp & 3, r = 32 * sub + lane, c0 = CE * ((warp - 6) >> 2);
+    const uint32_t lanes = tmem + ((uint32_t)(32 * sub) << 16) + (uint32_t)c0;
     while (!stop && it.next(cfg, set, i0, j0)) {
       WalkerDev& w = cfg.W[set >> 1];
-      const int sp = set & 1, n = w.n, ld = w.cap, b = (int)(k & 1u), i = i0 + r;
+      const int sp = set & 1, n = w.n, ld = w.cap, i = i0 + r;
       float* out = SECOND ? (float*)w.OzN[sp] : (float*)w.Ascr[sp];
       uint32_t dmax = 0u;
-      const bool mine = tc::mbar_wait(afull(b), (k >> 1) & 1u, abort_flag, cfg.wait_cycles);
-      if (!__all_sync(0xffffffffu, mine)) {
-        stop = true;
-        break;
-      }
-      tc::fence_after_sync();
-#pragma unroll 1
-      for (int cb = 0; cb < CB && j0 + cb < n; cb += 32) {
-        float v[32];
-        tc::tmem_ld32(tmem + ((uint32_t)(32 * sub) << 16) + (uint32_t)(CB * b + cb), v);
-        if (i < n) {
-          const size_t o = (size_t)i * ld + j0 + cb;  // 16-byte aligned: ld and j0 are multiples of 32
+      float acc[CE];
 #pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            const int j = j0 + cb + 4 * q;
-            if (j + 3 < n) {
-              *reinterpret_cast<float4*>(out + o + 4 * q) =
-                  make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-            } else {
+      for (int c = 0; c < CE; ++c) acc[c] = 0.0f;
+      for (int k0 = 0; k0 < n; k0 += 32, ++g) {
+        const int b = (int)(g & 1u);
+        const bool mine = tc::mbar_wait(afull(b), (g >> 1) & 1u, abort_flag, cfg.wait_cycles);
+        if (!__all_sync(0xffffffffu, mine)) {
+          stop = true;
+          break;
+        }
+        tc::fence_after_sync();
 #pragma unroll
-              for (int e = 0; e < 4; ++e)
-                if (j + e < n) out[o + 4 * q + e] = v[4 * q + e];
-            }
+        for (int cb = 0; cb < CE; cb += 32) {
+          float v[32];
+          tc::tmem_ld32(lanes + (uint32_t)(CB * b + cb), v);
 #pragma unroll
-            for (int e = 0; e < 4; ++e)
-              if (j + e < n) dmax = max(dmax, abs_bits(v[4 * q + e]));
+          for (int c = 0; c < 32; ++c) acc[cb + c] = __fadd_rn(acc[cb + c], v[c]);
+        }
+        if (k0 + 32 >= n) {
+#pragma unroll
+          for (int cb = 0; cb < CE; cb += 32) {
+            float v[32];
+            tc::tmem_ld32(lanes + (uint32_t)(2 * CB + CB * (int)(k & 1u) + cb), v);
+#pragma unroll
+            for (int c = 0; c < 32; ++c) acc[cb + c] = __fadd_rn(acc[cb + c], v[c]);
           }
         }
+        tc::fence_before_sync();
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(aempty(b));
       }
-      tc::fence_before_sync();
-      newton_max(&w.newton_bits[sp][SECOND ? 2 : 1], dmax);  // converges the warp
-      if (lane == 0) tc::mbar_arrive(aempty(b));
+      if (stop) break;
       ++k;
+      if (i < n) {
+        const size_t o = (size_t)i * ld + j0 + c0;  // 16-byte aligned: ld and j0 are multiples of 32
+#pragma unroll
+        for (int q = 0; q < CE / 4; ++q) {
+          const int j = j0 + c0 + 4 * q;
+          if (j + 3 < n) {
+            *reinterpret_cast<float4*>(out + o + 4 * q) =
+                make_float4(acc[4 * q], acc[4 * q + 1], acc[4 * q + 2], acc[4 * q + 3]);
+          } else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+              if (j + e < n) out[o + 4 * q + e] = acc[4 * q + e];
+          }
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (j + e < n) dmax = max(dmax, abs_bits(acc[4 * q + e]));
+        }
+      }
+      newton_max(&w.newton_bits[sp][SECOND ? 2 : 1], dmax);
     }
     if (stop && lane == 0) set_status(cfg.W[set >> 1], ST_ERR_TIMEOUT);
     if (stop) *abort_flag = 1;
@@ -315,8 +342,8 @@ cudaError_t setup_correct_tc() {
 }
 
 void launch_correct_tc(const Config& cfg, cudaStream_t st) {
-  k_correct_tc<false><<<device_sm_count(), 320, CoLayout::SMEM, st>>>(cfg);
-  k_correct_tc<true><<<device_sm_count(), 320, CoLayout::SMEM, st>>>(cfg);
+  k_correct_tc<false><<<device_sm_count(), CO_THREADS, CoLayout::SMEM, st>>>(cfg);
+  k_correct_tc<true><<<device_sm_count(), CO_THREADS, CoLayout::SMEM, st>>>(cfg);
 }
 
 }  // namespace dca
