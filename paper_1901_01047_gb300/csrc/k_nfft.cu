@@ -517,6 +517,10 @@ int launch_meas_nfft(const Config& cfg, int max_cap, int max_nc, cudaStream_t st
 
 static size_t nfft_finish_smem(int L) { return (size_t)L * (3 * sizeof(double2) + sizeof(double)); }
 
+size_t nfft_table_bytes(const Config& cfg) {
+  return cfg.freq_dft || nfft_finish_smem(cfg.nfft_L) > NFFT_FINISH_SMEM_MAX ? 0 : sizeof(double2) * 2 * (size_t)cfg.nfft_L;
+}
+
 void launch_nfft_table(const Config& cfg, double2* tab, cudaStream_t st) {
   k_nfft_table<<<(2 * cfg.nfft_L + 255) / 256, 256, 0, st>>>(cfg.nfft_L, tab);
 }

@@ -121,7 +121,9 @@ void launch_negate(const double* src, double* dst, float* dstf, size_t n, int* b
 // d_base, [2][nc][n_omega][re, im] each).
 cudaError_t setup_nfft();
 int launch_meas_nfft(const Config& cfg, int max_cap, int max_nc, cudaStream_t st);
-// tab: e^{i pi m / L}, m < 2L, filled once by launch_nfft_table.
+// tab: e^{i pi m / L}, m < 2L, filled once by launch_nfft_table; nfft_table_bytes is
+// 0 where the read-out does not use it.
+size_t nfft_table_bytes(const Config& cfg);
 void launch_nfft_table(const Config& cfg, double2* tab, cudaStream_t st);
 void launch_nfft_finish(const Config& cfg, int max_nc, const double2* tab, const long long* d_base, double* d_out,
                         cudaStream_t st);

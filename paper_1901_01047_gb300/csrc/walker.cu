@@ -20,6 +20,7 @@
 #include "../../include/dca_walker.h"
 #include "kernels.h"
 #include "problem_host.h"
+#include "readout.h"
 #include "state.h"
 
 using dca::ProblemDev;
@@ -94,6 +95,7 @@ struct dca_walker {
   bool g0_rejected = false;          // an update_G0 table had a non-finite entry (reported by sync)
   int64_t max_windows = 0;           // cap of the windows of one sweep call (0 = automatic)
   int prec_public = 0;               // DCA_PREC_* given at create
+  dca::ReadoutBuffers M_bufs, G_bufs;  // the buffers below
   double* d_Mout = nullptr;          // read-out of the frequency measurement, all walkers
   long long* d_Mbase = nullptr;      // its per-walker offsets
   double2* d_Mtab = nullptr;         // phases of the NFFT read-out
@@ -127,7 +129,10 @@ struct dca_walker {
 
   void* dalloc(size_t bytes) {
     void* p = nullptr;
-    if (cudaMalloc(&p, bytes ? bytes : 1) != cudaSuccess) return nullptr;
+    if (cudaMalloc(&p, bytes ? bytes : 1) != cudaSuccess) {
+      cudaGetLastError();  // reported by the caller, not again by its next launch
+      return nullptr;
+    }
     allocs.push_back(p);
     return p;
   }
@@ -1071,19 +1076,21 @@ extern "C" DCA_API int dca_walker_measure_G(dca_walker* h, double* G_out, double
     // every walker's accumulator gathered on the device into one buffer, one
     // copy to pinned host memory (instead of one small copy per walker)
     const size_t total = (size_t)h->gacc_off[h->W - 1] + (size_t)2 * h->nc_of[h->W - 1] * h->ntm;
-    if (!h->d_Gout) {
-      h->d_Gout = (double*)h->dalloc(sizeof(double) * total);
-      h->d_Gbase = (long long*)h->dalloc(sizeof(long long) * h->W);
-      if (!h->d_Gout || !h->d_Gbase) return fail(h, DCA_ERR_OOM, "read-out buffers of the tau-grid measurement");
-      if (cudaMallocHost(&h->h_Gout, sizeof(double) * total) != cudaSuccess) {
-        h->h_Gout = nullptr;
-        cudaGetLastError();
-        return fail(h, DCA_ERR_OOM, "pinned read-out buffer of the tau-grid measurement");
-      }
-      std::vector<long long> base(h->gacc_off.begin(), h->gacc_off.end());
-      CK(cudaMemcpyAsync(h->d_Gbase, base.data(), sizeof(long long) * h->W, cudaMemcpyHostToDevice, h->stream));
-      CK(cudaStreamSynchronize(h->stream));  // base is a host temporary
-    }
+    const int rb = h->G_bufs.prepare(
+        {{(void**)&h->d_Gout, sizeof(double) * total}, {(void**)&h->d_Gbase, sizeof(long long) * h->W}}, DCA_ERR_OOM,
+        [&](size_t bytes) { return h->dalloc(bytes); },
+        [&]() -> int {
+          if (!h->h_Gout && cudaMallocHost(&h->h_Gout, sizeof(double) * total) != cudaSuccess) {
+            h->h_Gout = nullptr;
+            cudaGetLastError();
+            return fail(h, DCA_ERR_OOM, "pinned read-out buffer of the tau-grid measurement");
+          }
+          std::vector<long long> base(h->gacc_off.begin(), h->gacc_off.end());
+          CK(cudaMemcpyAsync(h->d_Gbase, base.data(), sizeof(long long) * h->W, cudaMemcpyHostToDevice, h->stream));
+          CK(cudaStreamSynchronize(h->stream));  // base is a host temporary
+          return DCA_OK;
+        });
+    if (rb != DCA_OK) return h->G_bufs.base ? rb : fail(h, rb, "read-out buffers of the tau-grid measurement");
     dca::launch_gather_G(h->cfg, h->max_nc, h->d_Gbase, h->d_Gout, h->stream);
     h->total_launches += 1;
     CK(cudaGetLastError());
@@ -1114,15 +1121,18 @@ extern "C" DCA_API int dca_walker_measure_M(dca_walker* h, double* M_out, double
     total += per * h->nc_of[wi];
   }
   if (M_out) {
-    if (!h->d_Mout) {
-      h->d_Mout = (double*)h->dalloc(sizeof(double) * total);
-      h->d_Mbase = (long long*)h->dalloc(sizeof(long long) * h->W);
-      h->d_Mtab = (double2*)h->dalloc(sizeof(double2) * 2 * (size_t)h->cfg.nfft_L);
-      if (!h->d_Mout || !h->d_Mbase || !h->d_Mtab)
-        return fail(h, DCA_ERR_OOM, "read-out buffers of the frequency measurement");
-      CK(cudaMemcpyAsync(h->d_Mbase, base.data(), sizeof(long long) * h->W, cudaMemcpyHostToDevice, h->stream));
-      dca::launch_nfft_table(h->cfg, h->d_Mtab, h->stream);
-    }
+    const size_t table = dca::nfft_table_bytes(h->cfg);
+    const int rb = h->M_bufs.prepare(
+        {{(void**)&h->d_Mout, sizeof(double) * total}, {(void**)&h->d_Mbase, sizeof(long long) * h->W},
+         {(void**)&h->d_Mtab, table}}, DCA_ERR_OOM,
+        [&](size_t bytes) { return h->dalloc(bytes); },
+        [&]() -> int {
+          CK(cudaMemcpyAsync(h->d_Mbase, base.data(), sizeof(long long) * h->W, cudaMemcpyHostToDevice, h->stream));
+          if (table > 0) dca::launch_nfft_table(h->cfg, h->d_Mtab, h->stream);
+          CK(cudaGetLastError());
+          return DCA_OK;
+        });
+    if (rb != DCA_OK) return h->M_bufs.base ? rb : fail(h, rb, "read-out buffers of the frequency measurement");
     if (h->cfg.freq_dft) dca::launch_ndft_copy(h->cfg, h->max_nc, h->d_Mbase, h->d_Mout, h->stream);
     else dca::launch_nfft_finish(h->cfg, h->max_nc, h->d_Mtab, h->d_Mbase, h->d_Mout, h->stream);
     h->total_launches += 1;
