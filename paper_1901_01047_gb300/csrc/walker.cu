@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "../../include/dca_walker.h"
+#include "capture_guard.h"
 #include "kernels.h"
 #include "problem_host.h"
 #include "readout.h"
@@ -729,6 +730,18 @@ static int launch_window_sequence(dca_walker* h, const dca::Config& cfg, cudaStr
   return k;
 }
 
+// A capture of stream s into graph g, ended on every way out.
+static auto guard_capture(cudaStream_t s, cudaGraph_t g) {
+  auto begin = [=] { return cudaStreamBeginCaptureToGraph(s, g, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed); };
+  auto end = [=] {
+    cudaGraph_t captured = nullptr;
+    const cudaError_t e = cudaStreamEndCapture(s, &captured);
+    if (e != cudaSuccess) cudaGetLastError();  // reported by the caller, not again by its next launch
+    return e;
+  };
+  return dca::CaptureGuard<decltype(begin), decltype(end)>(begin, end);
+}
+
 // An IF node behind everything captured on cap_stream so far (a window body),
 // whose body is the given part of the window, of *kernels kernels.
 static int capture_if(dca_walker* h, const dca::Config& cfg, cudaGraphConditionalHandle handle, unsigned part, int* kernels) {
@@ -748,25 +761,27 @@ static int capture_if(dca_walker* h, const dca::Config& cfg, cudaGraphConditiona
   CK(cudaGraphAddNode(&node, g, deps, edges, nd, &np));
   CK(cudaStreamUpdateCaptureDependencies(h->cap_stream, &node, nullptr, 1, cudaStreamSetCaptureDependencies));
   if (!h->cap_br[0]) CK(cudaStreamCreateWithFlags(&h->cap_br[0], cudaStreamNonBlocking));
-  CK(cudaStreamBeginCaptureToGraph(h->cap_br[0], np.conditional.phGraph_out[0], nullptr, nullptr, 0,
-                                   cudaStreamCaptureModeRelaxed));
+  auto cap = guard_capture(h->cap_br[0], np.conditional.phGraph_out[0]);
+  CK(cap.start());
   *kernels = launch_window_sequence(h, cfg, h->cap_br[0], part);
-  cudaGraph_t captured = nullptr;
-  CK(cudaStreamEndCapture(h->cap_br[0], &captured));
+  CK(cap.finish());
   return DCA_OK;
 }
 
 // Build the device-side window loop once: an outer graph holding one
 // conditional WHILE node whose body (captured from the same launchers the
 // host loop uses) is one window plus the loop-control kernel.
-static int build_loop_graph(dca_walker* h) {
-  if (h->loop_exec) return DCA_OK;
+static int capture_loop(dca_walker* h) {
+  if (!h->h_loop && cudaMallocHost(&h->h_loop, sizeof(dca::LoopState)) != cudaSuccess) {
+    h->h_loop = nullptr;
+    cudaGetLastError();
+    return fail(h, DCA_ERR_OOM, "pinned loop state");
+  }
   if (!h->d_loop) {
-    h->d_loop = (dca::LoopState*)h->dalloc(sizeof(dca::LoopState));
-    if (!h->d_loop) return fail(h, DCA_ERR_OOM, "loop state allocation");
-    if (!h->h_loop && cudaMallocHost(&h->h_loop, sizeof(dca::LoopState)) != cudaSuccess)
-      return fail(h, DCA_ERR_OOM, "pinned loop state");
-    CK(cudaMemsetAsync(h->d_loop, 0, sizeof(dca::LoopState), h->stream));
+    dca::LoopState* state = (dca::LoopState*)h->dalloc(sizeof(dca::LoopState));
+    if (!state) return fail(h, DCA_ERR_OOM, "loop state allocation");
+    CK(cudaMemsetAsync(state, 0, sizeof(dca::LoopState), h->stream));
+    h->d_loop = state;  // zeroed, and its host copy is there: pull_records reads it from now on
   }
   if (!h->cap_stream) CK(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
   CK(cudaGraphCreate(&h->loop_graph, 0));
@@ -780,7 +795,8 @@ static int build_loop_graph(dca_walker* h) {
   cudaGraphNode_t node;
   CK(cudaGraphAddNode(&node, h->loop_graph, nullptr, nullptr, 0, &np));
   cudaGraph_t body = np.conditional.phGraph_out[0];
-  CK(cudaStreamBeginCaptureToGraph(h->cap_stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
+  auto cap = guard_capture(h->cap_stream, body);
+  CK(cap.start());
   int k = 0;
   const int nb = window_branches(h->W);
   if (nb > 1) {
@@ -833,12 +849,23 @@ static int build_loop_graph(dca_walker* h) {
   }
   dca::launch_loop_control(h->cfg, handle, h->d_loop, h->cap_stream);
   k += 1;
-  cudaGraph_t captured = nullptr;
-  cudaError_t e = cudaStreamEndCapture(h->cap_stream, &captured);
+  const cudaError_t e = cap.finish();
   if (e != cudaSuccess) return cuda_check(h, e, "capture of the window loop");
   CK(cudaGraphInstantiate(&h->loop_exec, h->loop_graph, 0));
   h->kernels_per_window = k;
   return DCA_OK;
+}
+
+static int build_loop_graph(dca_walker* h) {
+  if (h->loop_exec) return DCA_OK;
+  const int rc = capture_loop(h);
+  if (rc != DCA_OK) {  // nothing of it is left: the next sweep starts over
+    h->loop_exec = nullptr;
+    if (h->loop_graph) cudaGraphDestroy(h->loop_graph);
+    h->loop_graph = nullptr;
+    cudaGetLastError();
+  }
+  return rc;
 }
 
 // Enqueue n_sweeps of the device-side window loop: the sweep target, the
