@@ -87,6 +87,7 @@ constexpr int BA_R = 32, BA_C = 64;  // rows and columns of a k_build_A item
 // thread eight rows of a column.  Bound by the FP64 units (two lanes per SM).
 __global__ void __launch_bounds__(256) k_build_A(Config cfg, int mode) {
   __shared__ long long s_X[BA_R];
+  __shared__ double s_tau[BA_R];
   __shared__ int s_site[BA_R];
   if (blockIdx.x == 0 && threadIdx.x == 0) *cfg.gj_next = 0;  // work queue of the inverse that follows
   for_each_item(
@@ -106,12 +107,15 @@ __global__ void __launch_bounds__(256) k_build_A(Config cfg, int mode) {
         const bool pairs = mode == 1 && cfg.prec == PREC_MIXED && !cfg.recompute_gj;
         __syncthreads();  // the previous item of this block is done with the row records
         if (threadIdx.x < BA_R && i0 + threadIdx.x < n) {
-          s_X[threadIdx.x] = fixed_time(w.vtau[par][i0 + threadIdx.x], pb.tau_scale, F);
+          const double tau = w.vtau[par][i0 + threadIdx.x];
+          s_tau[threadIdx.x] = tau;
+          s_X[threadIdx.x] = fixed_time(tau, pb.tau_scale, F);
           s_site[threadIdx.x] = w.vsite[par][i0 + threadIdx.x];
         }
         __syncthreads();
         if (j >= n) return;
-        const long long Xj = fixed_time(w.vtau[par][j], pb.tau_scale, F), span = (long long)n_tau << F;
+        const double tau_j = w.vtau[par][j];
+        const long long Xj = fixed_time(tau_j, pb.tau_scale, F), span = (long long)n_tau << F;
         const int sj = w.vsite[par][j];
         const double ej = expV(pb, sp, w.vs[par][j]), mej1 = 1.0 - ej;
         const double* g0 = pb.g0 + (size_t)sp * nc * (size_t)(n_tau + 1);
@@ -121,10 +125,11 @@ __global__ void __launch_bounds__(256) k_build_A(Config cfg, int mode) {
           const int r = rl + (256 / BA_C) * u, i = i0 + r;
           if (i >= n) break;
           const double* row = g0 + (size_t)__ldg(pb.site_sub + s_site[r] * nc + sj) * (size_t)(n_tau + 1);
-          // g0(tau_i - tau_j): linear interpolation, g0(t - beta) = -g0(t), equal times read as 0+
+          // g0(tau_i - tau_j): linear interpolation, g0(t - beta) = -g0(t), equal times
+          // read as 0+ (times below 2^-62 beta of each other share a word: their order decides)
           long long D = s_X[r] - Xj;
           double m = mej1;
-          if (D < 0) {
+          if (D < 0 || (D == 0 && s_tau[r] < tau_j)) {
             D += span;
             m = __longlong_as_double(__double_as_longlong(m) ^ (1ll << 63));
           }
