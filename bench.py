@@ -62,13 +62,16 @@ MIXED_RECOMPUTE_TFLOPS = 4.0 / (2.0 / (FP32_INSTR_PER_S * 2 / 11 / 1e12) + 2.0 /
 # With the residual from digit planes on the tensor cores (the default), its
 # 2n^3 flop take 17 FP16 plane products of 2n^3 flop each at the measured
 # dense 16-bit tensor rate (the sustained BF16 figure: FP16 runs at the same
-# rate), the correction 2n^3 flop at the FP32 issue rate.
+# rate).  The correction's 2n^3 flop take three TF32 products on the tensor
+# cores, which is what the library runs ("tf32x3"), or one FMA per 2 flop at the
+# FP32 issue rate ("fp32").
 OZ_PRODUCTS = 17
 
 
-def sliced_recompute_tflops(peaks):
+def sliced_recompute_tflops(peaks, correction="fp32"):
     p16 = peaks.get("bf16_tflops_sustained", peaks["bf16_tflops"])
-    return 4.0 / (2.0 * OZ_PRODUCTS / p16 + 2.0 / (FP32_INSTR_PER_S * 2 / 1e12))
+    corr = {"fp32": 2.0 / (FP32_INSTR_PER_S * 2 / 1e12), "tf32x3": 6.0 / (p16 * TF32_PER_BF16)}[correction]
+    return 4.0 / (2.0 * OZ_PRODUCTS / p16 + corr)
 
 # DRAM bytes (read + write) per window of a kernel group from ncu captures of
 # the named workload (one window of the pooled schedule carries all walkers;
@@ -559,11 +562,12 @@ def run_ours(args, rank, world, local_rank):
     if rank == 0:
         peaks, kind = _peaks()
         windows = max(1, gtimes["propose"][1])  # one proposal kernel per window
-        roof = roofline(dominant, gtimes[dominant][0], windows, work, peaks, kind, wl)
+        roof = roofline(dominant, gtimes[dominant][0], windows, work, peaks, kind, wl, correction="tf32x3")
         roof_upd = roofline("update", gtimes["update"][0], windows, work, peaks, kind, wl)
         roof["traffic"] = NCU_TRAFFIC.get((wl.name, dominant))
         roof_upd["traffic"] = NCU_TRAFFIC.get((wl.name, "update"))
-        roof_rec = roofline("recompute", gtimes["recompute"][0], windows, work, peaks, kind, wl)
+        roof_rec = roofline("recompute", gtimes["recompute"][0], windows, work, peaks, kind, wl,
+                            correction="tf32x3")
         out = {
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": 1000.0 * seconds / args.steps, "higher_is_better": True,
@@ -619,10 +623,11 @@ def combine_ranks(dist, seconds, sums, device):
     return tuple(t.tolist())
 
 
-def roofline(group, g_ms, windows, work, peaks, kind, wl):
+def roofline(group, g_ms, windows, work, peaks, kind, wl, correction="fp32"):
     """Roofline of one kernel group from its CUDA-event time over the timed
     steps.  `work` maps a group to its algorithmic (bytes, flop) over the same
-    steps; the recompute counts flop only (FP64 arithmetic bound)."""
+    steps; the recompute counts flop only (FP64 arithmetic bound; `correction`:
+    the arithmetic of the default recompute's correction)."""
     sec = g_ms / 1000.0
     launch_ms = g_ms / max(1, windows)
     base = {"kernel": group, "launch_ms": launch_ms, "traffic": None}
@@ -633,11 +638,12 @@ def roofline(group, g_ms, windows, work, peaks, kind, wl):
     tfs = work_f / sec / 1e12
     if work_b is None:
         if wl.precision == "mixed" and wl.recompute_method == "auto":
-            pk = sliced_recompute_tflops(peaks)
+            pk = sliced_recompute_tflops(peaks, correction)
+            corr = {"fp32": "at the FP32 issue rate (152 SMs x 128 lanes x 2.07 GHz)",
+                    "tf32x3": "as 3 TF32 products at 1.1 / 2.25 of that rate"}[correction]
             return {**base, "bound": "tensor", "achieved": tfs, "peak": pk, "unit": "TFLOP/s", "frac": tfs / pk,
                     "peak_kind": "derived (%s): the residual's 2n^3 flop as %d FP16 plane products at the sustained "
-                                 "16-bit tensor rate, the correction's 2n^3 at the FP32 issue rate (152 SMs x 128 "
-                                 "lanes x 2.07 GHz)" % (kind, OZ_PRODUCTS)}
+                                 "16-bit tensor rate, the correction's 2n^3 %s" % (kind, OZ_PRODUCTS, corr)}
         if wl.precision == "mixed":
             return {**base, "bound": "alu", "achieved": tfs, "peak": MIXED_RECOMPUTE_TFLOPS, "unit": "TFLOP/s",
                     "frac": tfs / MIXED_RECOMPUTE_TFLOPS,
