@@ -36,7 +36,6 @@
 // come from one 64-bit integer product, and the phase (2n + 1) tau / beta
 // modulo 2 from another, so the sample loops of both variants run without
 // FP64 arithmetic (FP64 is 1/64 of the FP32 rate on this GPU).
-#include <algorithm>
 #include <cstdint>
 #include <type_traits>
 
@@ -247,10 +246,16 @@ __global__ void __launch_bounds__(256) k_meas_nfft(Config cfg) {
 // at a time, 24 lanes a sample, with plain loads and stores.  At the end of an
 // item (rb rows, dealt out over the warps) the grids are summed into the
 // walker's and cleared.  What is left is the FP64 work of the weights and the
-// load-add-store latency of a sample: 48 walkers of 4 sites, order 41, 64
-// frequencies, 240 -> 113 us a measurement.  (In FP32 the additions to shared memory
-// are cheap and the same layout was 2.5 times slower than k_meas_nfft.)
+// load-add-store latency of a sample.  The sum over the grids grows with them:
+// against k_meas_nfft a sweep's measurement took, at 48 walkers of 4 sites, order 47,
+// and 384 / 1024 / 2048 values a grid, 230 / 243 / 248 against 275 / 268 / 266 us;
+// of 8 sites, order 95, 768 / 2048 / 4096 values 872 / 925 / 1016 against 919 / 898 /
+// 889; 16 of 16 sites, order 54, 1536 / 4096 / 8192 values 279 / 311 / 337 against
+// 287 / 284 / 286.  Hence SPREAD_GRID: up to it never slower by more than 3 %, above
+// it mostly slower.  (In FP32 the additions to shared memory are cheap and the same
+// layout was 2.5 times slower than k_meas_nfft.)
 constexpr int SPREAD_WARPS = 8;
+constexpr size_t SPREAD_GRID = 1024;  // most values of a grid, spin up or down
 constexpr int SPREAD_WST = 33;  // odd stride of the weight rows
 constexpr size_t SPREAD_WEIGHT_BYTES = sizeof(double) * 2 * NFFT_MSP_MAX * SPREAD_WST;
 
@@ -455,6 +460,7 @@ __global__ void __launch_bounds__(256) k_nfft_finish_direct(Config cfg, const lo
 // accumulated in global memory directly.
 constexpr size_t NFFT_SMEM_MAX = 160 * 1024;
 constexpr size_t NFFT_SPREAD_SMEM_MAX = 220 * 1024;  // grids and weights of the FP64 spreading
+static_assert(SPREAD_WARPS * (sizeof(double) * SPREAD_GRID + SPREAD_WEIGHT_BYTES) <= NFFT_SPREAD_SMEM_MAX, "grids");
 constexpr size_t NFFT_FINISH_SMEM_MAX = 200 * 1024;  // tables of the read-out transform
 
 size_t nfft_smem_bytes(const Config& cfg, int max_nc) {
@@ -486,16 +492,13 @@ int launch_meas_nfft(const Config& cfg, int max_cap, int max_nc, cudaStream_t st
   if (cfg.freq_dft) return 1 + launch_meas_ndft(cfg, max_cap, max_nc, st);
   const long long items = 2LL * cfg.n_walkers * blocks_of(max_cap, NFFT_RB);
   const size_t smem = nfft_smem_bytes(cfg, max_nc);
-  // FP64: a grid per warp where at least two fit an SM's shared memory; larger
-  // grids (n_omega in the hundreds with 16 sites) are staged once per block or
-  // not at all.  Two rows a warp and item: the sum over the grids at its end
-  // costs about a fifth of a row.
-  const size_t per_warp = smem + SPREAD_WEIGHT_BYTES;
-  const int nw = (int)std::min<size_t>(SPREAD_WARPS, NFFT_SPREAD_SMEM_MAX / per_warp);
-  if (cfg.prec != PREC_MIXED && nw >= 2) {
-    const int per_sm = std::max(1, (int)(NFFT_SPREAD_SMEM_MAX / (nw * per_warp))), rb = 2 * nw;
+  // FP64: a grid per warp for small grids, larger ones staged once per block or
+  // not at all.  Two rows a warp and item.
+  if (cfg.prec != PREC_MIXED && (size_t)max_nc * cfg.nfft_L <= SPREAD_GRID) {
+    const size_t block = SPREAD_WARPS * (smem + SPREAD_WEIGHT_BYTES);
+    const int per_sm = (int)(NFFT_SPREAD_SMEM_MAX / block), rb = 2 * SPREAD_WARPS;
     const int grid = sm_grid(2LL * cfg.n_walkers * blocks_of(max_cap, rb), per_sm);
-    k_nfft_spread64<<<grid, 32 * nw, nw * per_warp, st>>>(cfg, rb, max_nc * cfg.nfft_L);
+    k_nfft_spread64<<<grid, 32 * SPREAD_WARPS, block, st>>>(cfg, rb, max_nc * cfg.nfft_L);
     return 2;
   }
   if (smem <= NFFT_SMEM_MAX) {
