@@ -47,8 +47,22 @@ namespace dca {
 
 // Rows of N per item.  A window measures a few walkers only, so the items have
 // to be many: with 64 rows two orders of 400 gave 28 blocks for 152 SMs (64
-// walkers, 128 frequencies, two measurements each: 3.85 -> 1.61 ms).
-constexpr int NFFT_RB = 16;
+// walkers, 128 frequencies, two measurements each: 3.85 -> 1.61 ms).  An item
+// clears and adds out its staged grid once, though: on the mixed path a grid of
+// 24576 values or more takes 32 rows where a lockstep batch measures all its walkers
+// at once (16 sites, 512 frequencies, order 340: a sweep's measurement of 8 / 24 / 64 /
+// 128 walkers 568 / 948 / 1857 / 3482 -> 530 / 919 / 1754 / 3231 us; at 16384 values
+// within 3 % either way; one walker 341 us with 16 rows, 457 with 64).  FP64, bound
+// by the additions, keeps 16: 32 rows are 6 to 15 % slower up to 38400 values.
+constexpr int NFFT_RB = 16, NFFT_RB_LARGE = 32;
+constexpr long long NFFT_LARGE_GRID = 24576;
+
+static int nfft_rows(const Config& cfg, int max_nc) {
+  const bool large = cfg.prec == PREC_MIXED && !cfg.pooled && cfg.n_walkers >= 8 &&
+                     (long long)max_nc * cfg.nfft_L >= NFFT_LARGE_GRID;
+  return large ? NFFT_RB_LARGE : NFFT_RB;
+}
+
 constexpr int NFFT_MSP_MAX = 12;
 constexpr unsigned long long X56_MASK = (1ull << 56) - 1ull;
 
@@ -169,13 +183,13 @@ __device__ __forceinline__ void spread_sample(S* g, int L, int msp, A a, const A
   }
 }
 
-// Item = (walker-spin, block of NFFT_RB rows of N); each warp takes every
+// Item = (walker-spin, block of rb rows of N); each warp takes every
 // eighth row of the block and its lanes stride over the columns.  SMEM: the
 // block stages the whole grid of its walker-spin (nc x L accumulators) in
 // shared memory and adds it to the walker's FP64 grid at the end of the item;
 // otherwise it adds every weight to the global grid directly.
 template <typename T, typename A, bool SMEM>
-__global__ void __launch_bounds__(256) k_meas_nfft(Config cfg) {
+__global__ void __launch_bounds__(256) k_meas_nfft(Config cfg, int rb) {
   extern __shared__ __align__(16) unsigned char nfft_raw[];
   __shared__ A s_e3[NFFT_MSP_MAX + 1];
   const int L = cfg.nfft_L, msp = cfg.nfft_msp;
@@ -186,7 +200,7 @@ __global__ void __launch_bounds__(256) k_meas_nfft(Config cfg) {
       2 * cfg.n_walkers,
       [&](int s) -> long long {
         const WalkerDev& w = cfg.W[s >> 1];
-        return wants_nfft(cfg, w) ? blocks_of(w.n, NFFT_RB) : 0;
+        return wants_nfft(cfg, w) ? blocks_of(w.n, rb) : 0;
       },
       [&](int s, int item) {
         const WalkerDev& w = cfg.W[s >> 1];
@@ -204,8 +218,8 @@ __global__ void __launch_bounds__(256) k_meas_nfft(Config cfg) {
           for (int e = threadIdx.x; e < nc * L; e += blockDim.x) g[e] = (S)0;
         __syncthreads();
         const double scale = w.sign / (pb.beta * (double)nc);
-        const int i0 = item * NFFT_RB;
-        const int i1 = min(n, i0 + NFFT_RB);
+        const int i0 = item * rb;
+        const int i1 = min(n, i0 + rb);
         for (int i = i0 + warp; i < i1; i += nwarps) {
           const unsigned long long wi = vx[i];
           if (wi == 0ull) continue;  // dead row: its factor e^{V} - 1 is zero
@@ -490,7 +504,8 @@ int launch_meas_nfft(const Config& cfg, int max_cap, int max_nc, cudaStream_t st
   k_freq_prep<<<cfg.n_walkers, 256, 0, st>>>(cfg);
   if (cfg.n_omega <= 0) return 1;
   if (cfg.freq_dft) return 1 + launch_meas_ndft(cfg, max_cap, max_nc, st);
-  const long long items = 2LL * cfg.n_walkers * blocks_of(max_cap, NFFT_RB);
+  const int rows = nfft_rows(cfg, max_nc);
+  const long long items = 2LL * cfg.n_walkers * blocks_of(max_cap, rows);
   const size_t smem = nfft_smem_bytes(cfg, max_nc);
   // FP64: a grid per warp for small grids, larger ones staged once per block or
   // not at all.  Two rows a warp and item.
@@ -504,16 +519,16 @@ int launch_meas_nfft(const Config& cfg, int max_cap, int max_nc, cudaStream_t st
   if (smem <= NFFT_SMEM_MAX) {
     if (cfg.prec == PREC_MIXED) {
       const void* fn = (const void*)k_meas_nfft<float, float, true>;
-      k_meas_nfft<float, float, true><<<persist_grid(fn, items, 256, smem), 256, smem, st>>>(cfg);
+      k_meas_nfft<float, float, true><<<persist_grid(fn, items, 256, smem), 256, smem, st>>>(cfg, rows);
     } else {
       const void* fn = (const void*)k_meas_nfft<double, double, true>;
-      k_meas_nfft<double, double, true><<<persist_grid(fn, items, 256, smem), 256, smem, st>>>(cfg);
+      k_meas_nfft<double, double, true><<<persist_grid(fn, items, 256, smem), 256, smem, st>>>(cfg, rows);
     }
   } else {
     if (cfg.prec == PREC_MIXED)
-      k_meas_nfft<float, float, false><<<sm_grid(items, 4), 256, 0, st>>>(cfg);
+      k_meas_nfft<float, float, false><<<sm_grid(items, 4), 256, 0, st>>>(cfg, rows);
     else
-      k_meas_nfft<double, double, false><<<sm_grid(items, 4), 256, 0, st>>>(cfg);
+      k_meas_nfft<double, double, false><<<sm_grid(items, 4), 256, 0, st>>>(cfg, rows);
   }
   return 2;
 }
