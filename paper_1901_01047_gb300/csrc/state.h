@@ -178,10 +178,12 @@ struct WalkerDev {
 __device__ __forceinline__ void set_status(WalkerDev& w, int32_t code) { atomicCAS(&w.status, (int32_t)ST_OK, code); }
 
 // Whether the Newton recompute of a walker-spin takes its second term N0 R^2
-// (k_refine.cu): max |R| from NEWTON_R_MIN on, where what one term leaves reaches
-// the FP32 rounding of N, and below 1, past which the series does not converge
-// (NaN and infinity order above).
-constexpr float NEWTON_R_MIN = 1e-4f;
+// (k_refine.cu): max |R| from NEWTON_R_MIN on, and below 1, past which the series
+// does not converge (NaN and infinity order above).  What one term leaves of G is
+// about R^2 there (16 sites, beta = 16: 1.8e-7 at 4.5e-4 beside 1.9e-7 of the FP32
+// rounding), so 6e-8 at the line; from 1e-4 on the second term would cost the batch
+// of 256 2.3 % of a pass, from 2.5e-4 on 1.6 %, from 5e-4 on 0.9 %.
+constexpr float NEWTON_R_MIN = 2.5e-4f;
 __device__ __forceinline__ bool newton_second(const WalkerDev& w, int sp) {
   return w.newton_bits[sp][0] >= __float_as_uint(NEWTON_R_MIN) && w.newton_bits[sp][0] < __float_as_uint(1.0f);
 }
