@@ -4,7 +4,7 @@
 // interpolated on the fly while tiles of MK vertices pass through shared
 // memory, so a tile costs one interpolation per (x, a, i) and nc products of
 // it; the work item is a site x, a block of tau points and all vertices of one
-// walker-spin.
+// walker-spin (or VSEG of them).
 #include <cstdint>
 
 #include "device_util.cuh"
@@ -18,13 +18,17 @@ namespace {
 constexpr int MK = 32;    // vertices per tile
 constexpr int MT = 128;   // tau points per item, FP32 kernel
 constexpr int AST = MT + 4;
-// Vertices per item of the FP32 kernel for up to 16 sites: a window measures a
-// few walkers only, and one of 16 sites with 256 tau points is 64 items without
-// this split (a measurement of 16 sites, order 640, 114 -> 76 us).  Larger clusters
-// have items enough, and the split costs 4 of 36 sites 7 % of a sweep.
-template <int CLASS>
+// Vertices per item of the FP32 kernel (SPLIT) where the items of a measurement are
+// fewer than the SMs without it: one walker of 16 sites with 256 tau points is 64
+// items (order 640, 114 -> 76 us; a sweep's measurement with 32 / 128 items, order 408,
+// 230 / 244 -> 216 / 233 us, one of 36 sites, 72 items, 300 -> 281).  With items enough
+// the split only adds flushes and atomics: 256 / 768 / 12288 items of 16 sites 252 /
+// 400 / 2326 -> 267 / 438 / 3044 us, 576 of 36 sites 458 -> 491.  Clusters above 36
+// sites, one block an SM, lose from 98 items on.
+constexpr int VSEG = 256, VSEG_ITEMS = 152;
+template <bool SPLIT>
 __host__ __device__ constexpr int vseg() {
-  return CLASS == 0 ? 256 : 1 << 30;
+  return SPLIT ? VSEG : 1 << 30;
 }
 constexpr int DT = 16;    // tau points per item, FP64 kernel
 
@@ -78,7 +82,7 @@ __device__ __forceinline__ void df_add(float& hi, float& lo, float x) {
   hi = s;
 }
 
-template <int CLASS, int NG, int SR, int TA>
+template <bool SPLIT, int NG, int SR, int TA>
 __device__ __forceinline__ void meas_item_f(const Config& cfg, const WalkerDev& w, int sp, int item, MeasSmem& sm,
                                             float* dyn) {
   constexpr int TT = MT / TA;            // tau threads
@@ -89,7 +93,7 @@ __device__ __forceinline__ void meas_item_f(const Config& cfg, const WalkerDev& 
   constexpr int BST = bs_stride<NG, SR>();
   const ProblemDev& pb = cfg.P[w.problem];
   const int nc = pb.nc, ntm = cfg.n_tau_meas, par = w.parity, ld = w.cap, q = pb.meas_q;
-  constexpr int VS = vseg<CLASS>();
+  constexpr int VS = vseg<SPLIT>();
   const int tblocks = (ntm + MT - 1) / MT, segs = (int)blocks_of(w.n, VS);
   const int v0 = (item % segs) * VS, n = (int)min((long long)w.n, (long long)v0 + VS);  // the item's vertices v0 .. n - 1
   item /= segs;
@@ -272,7 +276,7 @@ __device__ __forceinline__ void meas_item_f(const Config& cfg, const WalkerDev& 
 
 }  // namespace
 
-template <int CLASS>
+template <int CLASS, bool SPLIT>
 __global__ void __launch_bounds__(256, CLASS == 2 ? 1 : 2) k_meas_gemm(Config cfg) {
   extern __shared__ __align__(16) float dyn[];
   __shared__ MeasSmem sm;
@@ -282,17 +286,17 @@ __global__ void __launch_bounds__(256, CLASS == 2 ? 1 : 2) k_meas_gemm(Config cf
         const WalkerDev& w = cfg.W[s >> 1];
         const int nc = cfg.P[w.problem].nc;
         return (wants_gemm(w) && site_class(nc) == CLASS)
-                   ? (long long)nc * blocks_of(cfg.n_tau_meas, MT) * blocks_of(w.n, vseg<CLASS>()) : 0;
+                   ? (long long)nc * blocks_of(cfg.n_tau_meas, MT) * blocks_of(w.n, vseg<SPLIT>()) : 0;
       },
       [&](int s, int item) {
         const WalkerDev& w = cfg.W[s >> 1];
         if constexpr (CLASS == 0) {
-          if (cfg.P[w.problem].nc <= 8) meas_item_f<CLASS, 2, 4, 4>(cfg, w, s & 1, item, sm, dyn);
-          else meas_item_f<CLASS, 4, 4, 4>(cfg, w, s & 1, item, sm, dyn);
+          if (cfg.P[w.problem].nc <= 8) meas_item_f<SPLIT, 2, 4, 4>(cfg, w, s & 1, item, sm, dyn);
+          else meas_item_f<SPLIT, 4, 4, 4>(cfg, w, s & 1, item, sm, dyn);
         } else if constexpr (CLASS == 1) {
-          meas_item_f<CLASS, 4, 9, 2>(cfg, w, s & 1, item, sm, dyn);
+          meas_item_f<SPLIT, 4, 9, 2>(cfg, w, s & 1, item, sm, dyn);
         } else {
-          meas_item_f<CLASS, 4, 16, 2>(cfg, w, s & 1, item, sm, dyn);
+          meas_item_f<SPLIT, 4, 16, 2>(cfg, w, s & 1, item, sm, dyn);
         }
       });
 }
@@ -405,25 +409,41 @@ __global__ void __launch_bounds__(256) k_meas_gemm64(Config cfg) {
 }
 
 cudaError_t setup_meas_gemm() {
-  cudaError_t e = cudaFuncSetAttribute(k_meas_gemm<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_class(0));
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_meas_gemm<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_class(1));
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_meas_gemm<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_class(2));
+  cudaError_t e = cudaSuccess;
+  auto set = [&](const void* fn, int c) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_class(c));
+  };
+  set((const void*)k_meas_gemm<0, false>, 0);
+  set((const void*)k_meas_gemm<0, true>, 0);
+  set((const void*)k_meas_gemm<1, false>, 1);
+  set((const void*)k_meas_gemm<1, true>, 1);
+  set((const void*)k_meas_gemm<2, false>, 2);
   return e;
 }
 
-template <int CLASS>
+template <int CLASS, bool SPLIT>
 static void gemm_f(const Config& cfg, long long items, cudaStream_t st) {
   constexpr int sm = smem_class(CLASS);
-  k_meas_gemm<CLASS><<<persist_grid((const void*)k_meas_gemm<CLASS>, items, 256, sm), 256, sm, st>>>(cfg);
+  const void* fn = (const void*)k_meas_gemm<CLASS, SPLIT>;
+  k_meas_gemm<CLASS, SPLIT><<<persist_grid(fn, items, 256, sm), 256, sm, st>>>(cfg);
 }
 
 int launch_meas_gemm(const Config& cfg, int max_cap, int max_nc, cudaStream_t st) {
   const long long S = 2LL * cfg.n_walkers;
   if (cfg.prec == PREC_MIXED) {
     const long long items = S * max_nc * blocks_of(cfg.n_tau_meas, MT);
-    gemm_f<0>(cfg, items * blocks_of(max_cap, vseg<0>()), st);
-    if (max_nc > 16) gemm_f<1>(cfg, items, st);
-    if (max_nc > 36) gemm_f<2>(cfg, items, st);
+    // walkers that measure in one window: all under the lockstep schedule, else about
+    // one of the windows that a sweep takes
+    const long long at_once = cfg.pooled ? blocks_of(cfg.n_walkers, 8) : cfg.n_walkers;
+    auto split = [&](int nc) { return 2 * at_once * nc * blocks_of(cfg.n_tau_meas, MT) < VSEG_ITEMS; };
+    const long long parts = items * blocks_of(max_cap, VSEG);
+    if (split(max_nc < 16 ? max_nc : 16)) gemm_f<0, true>(cfg, parts, st);
+    else gemm_f<0, false>(cfg, items, st);
+    if (max_nc > 16) {
+      if (split(max_nc < 36 ? max_nc : 36)) gemm_f<1, true>(cfg, parts, st);
+      else gemm_f<1, false>(cfg, items, st);
+    }
+    if (max_nc > 36) gemm_f<2, false>(cfg, items, st);
     return 1 + (max_nc > 16) + (max_nc > 36);
   }
   const long long items = S * max_nc * blocks_of(cfg.n_tau_meas, DT);
