@@ -2,7 +2,7 @@
 // cluster per matrix (the from-scratch N of the initial build and of the
 // periodic recompute, Eq. Zk: N = [e^V - g0 (e^V - 1)]^-1).
 //
-// A cluster of C blocks (16 for a few matrices, else 8) shares one n x n
+// A cluster of C blocks (16 for up to 6 matrices, else 8) shares one n x n
 // matrix in global memory; row r belongs to block r % C.  The columns are taken
 // in panels of B.  With J the rows of a panel after its row interchanges,
 //   A_JJ <- A_JJ^-1,  A_Jk <- A_JJ^-1 A_Jk,  A_iJ <- -A_iJ A_JJ^-1,
@@ -43,6 +43,7 @@ namespace {
 
 constexpr int GJ_THREADS = 1024;
 constexpr int GJ_MAX_CTAS = 16;
+constexpr int GJ_WIDE_MATS = 6;        // most matrices for clusters of 16
 constexpr int GJ_XC = 256;             // columns of X in shared memory at a time
 constexpr size_t GJ_SMEM = 208 * 1024;  // dynamic shared memory of a block, at most
 
@@ -475,13 +476,13 @@ cudaError_t gj_launch(const Config& cfg, int mode, int max_n, int ctas, int clus
   return cudaLaunchKernelEx(&lc, k_gj_cluster<B>, cfg, mode, max_n, work, d_sgn);
 }
 
-// Kernel attributes (once per device) and whether a cluster of 16 fits the device.
+// Kernel attributes (once per device) and the clusters of 16 that the device holds at once.
 template <int B>
-bool gj_setup() {
+int gj_setup() {
   cudaFuncSetAttribute(k_gj_cluster<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GJ_SMEM);
   if (cudaFuncSetAttribute(k_gj_cluster<B>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
     cudaGetLastError();
-    return false;
+    return 0;
   }
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3(GJ_MAX_CTAS);
@@ -497,9 +498,9 @@ bool gj_setup() {
   int got = 0;
   if (cudaOccupancyMaxActiveClusters(&got, k_gj_cluster<B>, &lc) != cudaSuccess) {
     cudaGetLastError();
-    return false;
+    return 0;
   }
-  return got > 0;
+  return got;
 }
 
 size_t gw_smem(int n) { return sizeof(double) * (size_t)gj_rows(n, GJ_MAX_CTAS) * (GW_B + 1); }
@@ -563,28 +564,31 @@ bool launch_gj_wide(const Config& cfg, int n, int* d_sgn, cudaStream_t st) {
 
 void launch_gj(const Config& cfg, int mode, int max_n, int* d_sgn, cudaStream_t st) {
   static std::mutex mu;
-  static int state[64] = {0};  // per device: 0 unknown, 1 clusters of 8 only, 2 clusters of 16 too
+  static int state[64] = {0};  // per device: 0 unknown, else 1 + the clusters of 16 it holds
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) dev = 0;
-  bool wide;
+  int wide;
   {
     std::lock_guard<std::mutex> lk(mu);
     if (state[dev] == 0) {
-      const bool a = gj_setup<16>();
+      const int a = gj_setup<16>();
       gj_setup<4>();
       gj_setup<1>();
-      state[dev] = a ? 2 : 1;
+      state[dev] = 1 + a;
     }
-    wide = state[dev] == 2;
+    wide = state[dev] - 1;
   }
   if (max_n < 1) max_n = 1;
   const int mats = 2 * cfg.n_walkers;
   // Panels of 16 columns while the panel rows of a block fit beside X (n up to
-  // about 9000 on 8 blocks), else of 4 (about 40000) or single columns.  Few
-  // matrices take clusters of 16 blocks, so that one matrix has the FP64 units
-  // of 16 SMs (eight such clusters fit); more matrices clusters of 8 on all SMs.
+  // about 9000 on 8 blocks), else of 4 (about 40000) or single columns.  Up to
+  // GJ_WIDE_MATS matrices take clusters of 16 blocks, so that one matrix has the
+  // FP64 units of 16 SMs; more take clusters of 8 on all SMs, a second wave of
+  // the larger ones being slower: a sweep's recompute of 2 / 6 / 8 / 10 matrices of
+  // order 310 1478 / 1596 / 2744 / 2839 us on clusters of 16, 2119 / 2328 / 2406 / 2407
+  // on 8; of order 50 262 / - / 383 / 586 against 272 / - / 272 / 477.
   auto fits = [&](int c, int B) { return gj_rp_bytes(max_n, B) + gj_work_bytes(gj_rows(max_n, c), B) <= GJ_SMEM; };
-  const int ctas = wide && mats <= 8 && fits(GJ_MAX_CTAS, 16) ? GJ_MAX_CTAS : 8;
+  const int ctas = mats <= wide && mats <= GJ_WIDE_MATS && fits(GJ_MAX_CTAS, 16) ? GJ_MAX_CTAS : 8;
   const int fit = device_sm_count() / ctas > 0 ? device_sm_count() / ctas : 1;
   const int clusters = mats < fit ? mats : fit;
   if (fits(ctas, 16)) gj_launch<16>(cfg, mode, max_n, ctas, clusters, d_sgn, st);

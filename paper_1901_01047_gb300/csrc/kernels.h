@@ -61,7 +61,7 @@ void launch_fresh_inverse(const Config& cfg, int max_n, int* d_sgn, cudaStream_t
 // (nothing launched) where the order or the device is better served by launch_gj.
 size_t gj_wide_scratch(int n);
 bool launch_gj_wide(const Config& cfg, int n, int* d_sgn, cudaStream_t st);
-// Gauss-Jordan inverse of the FP64 work matrices, one 8-block cluster each.
+// Gauss-Jordan inverse of the FP64 work matrices, one cluster of 8 or 16 blocks each.
 void launch_gj(const Config& cfg, int mode, int max_n, int* d_sgn, cudaStream_t st);
 // Mixed-precision recompute by a Newton step against the FP64 A = N^-1: the
 // products (R = I - A N0 in FP64, N0 R in FP32 and where R is large N0 R^2), then
