@@ -355,36 +355,26 @@ __global__ void __launch_bounds__(256, 3) k_cand_cc(Config cfg) {
 // ---------------------------------------------------------------------------
 // Metropolis over the window (one block per walker, both spins).
 // ---------------------------------------------------------------------------
-// Arithmetic M of the bordered growth of B^-1 and of the Schur complements
-// (the determinant ratios): FP64 (double), or double-float pairs (hi, lo) of
-// FP32 (float2), about 44 significant bits at the FP32 issue rate.  The
-// update kernels of the mixed path read B^-1 as such pairs, so the FP64
-// variant on the mixed path converts B^-1 into them at the end of the window.
+// Arithmetic of the bordered growth of B^-1 and of the Schur complements (the
+// determinant ratios) here: double-float pairs (hi, lo) of FP32, about 44
+// significant bits at the FP32 issue rate, the form in which the update kernels
+// of the mixed path read B^-1.
 
-__device__ __forceinline__ void m_set(double& r, double x) { r = x; }
 __device__ __forceinline__ void m_set(float2& r, double x) { r = df_split(x); }
-__device__ __forceinline__ double m_val(double a) { return a; }
 __device__ __forceinline__ double m_val(float2 a) { return (double)a.x + (double)a.y; }
-__device__ __forceinline__ void m_zero(double& a) { a = 0.0; }
 __device__ __forceinline__ void m_zero(float2& a) { a = make_float2(0.f, 0.f); }
 // acc += a b
-__device__ __forceinline__ void m_fma(double& acc, double a, double b) { acc = fma(a, b, acc); }
 __device__ __forceinline__ void m_fma(float2& acc, float2 a, float2 b) { df_fma(acc.x, acc.y, a.x, a.y, b.x, b.y); }
 // acc += b
-__device__ __forceinline__ void m_acc(double& acc, double b) { acc += b; }
 __device__ __forceinline__ void m_acc(float2& acc, float2 b) { df_fma(acc.x, acc.y, b.x, b.y, 1.f, 0.f); }
 // normalised value of an accumulator
-__device__ __forceinline__ double m_fin(double a) { return a; }
 __device__ __forceinline__ float2 m_fin(float2 a) { return df_norm(a.x, a.y); }
-__device__ __forceinline__ double m_neg(double a) { return -a; }
 __device__ __forceinline__ float2 m_neg(float2 a) { return make_float2(-a.x, -a.y); }
-__device__ __forceinline__ double m_mul(double a, double b) { return a * b; }
 __device__ __forceinline__ float2 m_mul(float2 a, float2 b) {
   float hi = 0.f, lo = 0.f;
   df_fma(hi, lo, a.x, a.y, b.x, b.y);
   return df_norm(hi, lo);
 }
-__device__ __forceinline__ double m_shfl_xor(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
 __device__ __forceinline__ float2 m_shfl_xor(float2 a, int o) {
   return make_float2(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o));
 }
@@ -406,7 +396,6 @@ __device__ __forceinline__ int row_lanes(int l) {
 // and (7) the bordered inverse [[B^-1 + t s, -t / d], [-s, 1 / d]].  Thread 0
 // plans proposal j + 1 (step 1) together with decision j, so a rejection
 // costs three block barriers and an acceptance four.
-template <typename T, typename M>
 __global__ void __launch_bounds__(256) k_metropolis(Config cfg) {
   WalkerDev& w = cfg.W[blockIdx.x];
   __shared__ int s_active;
@@ -416,7 +405,7 @@ __global__ void __launch_bounds__(256) k_metropolis(Config cfg) {
   const ProblemDev& pb = cfg.P[w.problem];
   const int tid = threadIdx.x;
   const int n = w.n, n_live = w.n_live, len = w.win_len;
-  const ExtView<T> ev[2] = {make_view<T>(w, 0), make_view<T>(w, 1)};
+  const ExtView<float> ev[2] = {make_view<float>(w, 0), make_view<float>(w, 1)};
   // B^-1 of both spins: in shared memory when k_s <= METRO_SMEM_KS, with row
   // stride k_s | 1 (odd: the row-wise products of step 3 are free of bank
   // conflicts), copied to the global buffers at the end; else in the global
@@ -424,13 +413,14 @@ __global__ void __launch_bounds__(256) k_metropolis(Config cfg) {
   extern __shared__ double s_binv[];
   const bool in_smem = cfg.ks <= METRO_SMEM_KS;
   const int bst = in_smem ? (cfg.ks | 1) : KS_MAX;
-  M* const Binv[2] = {in_smem ? reinterpret_cast<M*>(s_binv) : reinterpret_cast<M*>(w.Binv[0]),
-                      in_smem ? reinterpret_cast<M*>(s_binv) + (size_t)cfg.ks * bst : reinterpret_cast<M*>(w.Binv[1])};
+  float2* const Binv[2] = {in_smem ? reinterpret_cast<float2*>(s_binv) : reinterpret_cast<float2*>(w.Binv[0]),
+                           in_smem ? reinterpret_cast<float2*>(s_binv) + (size_t)cfg.ks * bst
+                                   : reinterpret_cast<float2*>(w.Binv[1])};
 
   __shared__ Proposal s_prop[KS_MAX];
   __shared__ int s_live[METRO_LIVE];  // 2 row + (s > 0) of the live vertex of each rank
-  __shared__ M s_brow[2][KS_MAX], s_bcol[2][KS_MAX], s_t[2][KS_MAX], s_s[2][KS_MAX];
-  __shared__ M s_rd[2];
+  __shared__ float2 s_brow[2][KS_MAX], s_bcol[2][KS_MAX], s_t[2][KS_MAX], s_s[2][KS_MAX];
+  __shared__ float2 s_rd[2];
   __shared__ double s_aP[2][KS_MAX];
   __shared__ int s_P[KS_MAX];
   __shared__ int s_Pup[KS_MAX];       // spin of a live P_p > 0
@@ -651,7 +641,7 @@ __global__ void __launch_bounds__(256) k_metropolis(Config cfg) {
         const int qp = s_upq;
         for (int idx = tid; idx < 2 * l; idx += blockDim.x) {
           const int sp = idx >= l ? 1 : 0, i = idx - sp * l;
-          const M* B = Binv[sp];
+          const float2* B = Binv[sp];
           m_set(s_t[sp][i], -m_val(s_rd[sp]) * ((i == qp ? 1.0 : 0.0) - m_val(B[(size_t)i * bst + qp])));
           s_s[sp][i] = B[(size_t)qp * bst + i];
         }
@@ -659,8 +649,8 @@ __global__ void __launch_bounds__(256) k_metropolis(Config cfg) {
         for (int idx = tid; idx < 2 * l * l; idx += blockDim.x) {
           const int sp = idx >= l * l ? 1 : 0, r = idx - sp * l * l;
           const int i = r / l, jj = r - i * l;
-          M* B = Binv[sp] + (size_t)i * bst + jj;
-          M b = *B;
+          float2* B = Binv[sp] + (size_t)i * bst + jj;
+          float2 b = *B;
           m_fma(b, s_t[sp][i], s_s[sp][jj]);
           *B = m_fin(b);
         }
@@ -699,10 +689,10 @@ __global__ void __launch_bounds__(256) k_metropolis(Config cfg) {
       const int r = tid / G, g = tid - r * G;
       const bool ok = r < 2 * l;
       const int sp = ok ? r / l : 0, i = ok ? r - sp * l : 0;
-      M acc;
+      float2 acc;
       m_zero(acc);
       if (ok) {
-        const M* B = Binv[sp] + (size_t)i * bst;
+        const float2* B = Binv[sp] + (size_t)i * bst;
         for (int p = g; p < l; p += G) m_fma(acc, B[p], s_bcol[sp][p]);
       }
       for (int o = G >> 1; o > 0; o >>= 1) m_acc(acc, m_shfl_xor(acc, o));
@@ -712,7 +702,7 @@ __global__ void __launch_bounds__(256) k_metropolis(Config cfg) {
     // 4. Schur complements d = B_tt - b_row . t, and 5. the decision (warp 0);
     //    thread 0 then records an acceptance and plans proposal j + 1
     if (tid < 32) {
-      M a0, a1;
+      float2 a0, a1;
       m_zero(a0);
       m_zero(a1);
       for (int i = tid; i < l; i += 32) {
@@ -818,7 +808,7 @@ __global__ void __launch_bounds__(256) k_metropolis(Config cfg) {
       const int r = tid / G, g = tid - r * G;
       const bool ok = r < 2 * l;
       const int sp = ok ? r / l : 0, jj = ok ? r - sp * l : 0;
-      M acc;
+      float2 acc;
       m_zero(acc);
       if (ok)
         for (int i = g; i < l; i += G) m_fma(acc, s_brow[sp][i], Binv[sp][(size_t)i * bst + jj]);
@@ -832,9 +822,9 @@ __global__ void __launch_bounds__(256) k_metropolis(Config cfg) {
       for (int idx = tid; idx < 2 * e; idx += blockDim.x) {
         const int sp = idx >= e ? 1 : 0, r = idx - sp * e;
         const int i = r / (l + 1), jj = r - i * (l + 1);
-        M* B = Binv[sp] + (size_t)i * bst + jj;
+        float2* B = Binv[sp] + (size_t)i * bst + jj;
         if (i < l && jj < l) {
-          M b = *B;
+          float2 b = *B;
           m_fma(b, s_t[sp][i], s_s[sp][jj]);
           *B = m_fin(b);
         } else if (i < l) {
@@ -853,17 +843,12 @@ __global__ void __launch_bounds__(256) k_metropolis(Config cfg) {
 
   // Epilogue: window bookkeeping and the accepted set.
   const int l = s_l, nrem = s_nrem, nins = s_nins, nflip = s_nflip;
-  // B^-1 for the update kernels: FP64 on the FP64 path, FP32 pairs on the
-  // mixed path (converted in place, element by element, when the growth ran
-  // in FP64 in the global buffer)
-  constexpr bool to_pairs = sizeof(T) == 4 && sizeof(M) == 8 && !std::is_same<M, float2>::value;
-  if (in_smem || to_pairs)
+  // B^-1 for the update kernels
+  if (in_smem)
     for (int sp = 0; sp < 2; ++sp)
       for (int idx = tid; idx < l * l; idx += blockDim.x) {
         const int i = idx / l, jj = idx - i * l;
-        const M b = Binv[sp][(size_t)i * bst + jj];
-        if (to_pairs) reinterpret_cast<float2*>(w.Binv[sp])[(size_t)i * KS_MAX + jj] = df_split(m_val(b));
-        else reinterpret_cast<M*>(w.Binv[sp])[(size_t)i * KS_MAX + jj] = b;
+        reinterpret_cast<float2*>(w.Binv[sp])[(size_t)i * KS_MAX + jj] = Binv[sp][(size_t)i * bst + jj];
       }
   for (int p = tid; p < l; p += blockDim.x) {
     w.P[p] = s_P[p];
@@ -1075,11 +1060,10 @@ __device__ __forceinline__ void upd_apply_tile(const Config& cfg, int wi, int sp
 //   N[i, n+m']   = Lp[i, p(c_m')]                                (i < n)
 //   N[n+m, n+m'] = delta + Lp[n+c_m, p(c_m')]
 // (R[p, n+c] is 1 only where P_p is candidate c itself.)
-template <typename T, typename A>
-__global__ void __launch_bounds__(256) k_upd_border(Config cfg) {
+__global__ void __launch_bounds__(256) k_upd_border(Config cfg) {  // tensor-core update: FP32
   for_each_item(
       2 * cfg.n_walkers, [&](int s) -> long long { return border_items(cfg.W[s >> 1]); },
-      [&](int s, int item) { upd_border_item<T, A>(cfg, s >> 1, s & 1, item); });
+      [&](int s, int item) { upd_border_item<float, float>(cfg, s >> 1, s & 1, item); });
 }
 
 template <typename T, typename A>
@@ -1419,7 +1403,7 @@ static int launch_group_t(int group, const Config& cfg, int max_cap, cudaStream_
         launch_metropolis64(cfg, st);
       } else {
         const int sm = cfg.ks <= METRO_SMEM_KS ? (int)sizeof(double) * 2 * cfg.ks * (cfg.ks | 1) : 0;
-        k_metropolis<float, float2><<<W, 256, sm, st>>>(cfg);
+        k_metropolis<<<W, 256, sm, st>>>(cfg);
       }
       return 1;
     }
@@ -1439,8 +1423,7 @@ static int launch_group_t(int group, const Config& cfg, int max_cap, cudaStream_
     case GROUP_UPDATE_POST:
       // (the CUDA-core update has done the insertions' rows and columns)
       if (sizeof(T) == 4 && cfg.upd_kernel == UPD_TCGEN05)
-        k_upd_border<float, float><<<persist_grid((const void*)k_upd_border<float, float>, 2 * S * kc, 256), 256, 0,
-                                     st>>>(cfg);
+        k_upd_border<<<persist_grid((const void*)k_upd_border, 2 * S * kc, 256), 256, 0, st>>>(cfg);
       k_window_end<<<W, 256, 0, st>>>(cfg);
       k_compact_N<T><<<persist_grid((const void*)k_compact_N<T>, S * t32 * t32, 256), 256, 0, st>>>(cfg);
       k_compact_end<<<W, 256, 0, st>>>(cfg);
@@ -1455,7 +1438,7 @@ cudaError_t setup_window_kernels() {
   const int msm = (int)sizeof(double) * 2 * METRO_SMEM_KS * (METRO_SMEM_KS | 1);
   cudaError_t e = setup_metropolis64();
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_metropolis<float, float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, msm);
+    e = cudaFuncSetAttribute(k_metropolis, cudaFuncAttributeMaxDynamicSharedMemorySize, msm);
   return e;
 }
 
