@@ -53,8 +53,8 @@ constexpr size_t kOffSpin = kOffTau + up256(sizeof(double) * kMaxOrder);
 constexpr size_t kOffN0 = kOffSpin + up256(sizeof(int32_t) * kMaxOrder);
 constexpr size_t kOffN1 = kOffN0 + up256(sizeof(double) * kMaxOrder * kMaxOrder);
 constexpr size_t kOffScr0 = kOffN1 + up256(sizeof(double) * kMaxOrder * kMaxOrder);
-constexpr size_t kOffScr1 = kOffScr0 + up256(sizeof(double) * 16 * kMaxOrder);
-constexpr size_t kOffSign = kOffScr1 + up256(sizeof(double) * 16 * kMaxOrder);
+constexpr size_t kOffScr1 = kOffScr0 + up256(sizeof(double) * dca::GJ_X_ROWS * kMaxOrder);
+constexpr size_t kOffSign = kOffScr1 + up256(sizeof(double) * dca::GJ_X_ROWS * kMaxOrder);
 constexpr size_t kScratchBytes = kOffSign + up256(sizeof(int32_t) * 4);  // two signs, work queue
 
 static __device__ __align__(256) unsigned char g_fresh_scratch[kScratchBytes];
@@ -125,8 +125,8 @@ extern "C" DCA_API int dca_fresh_N_noalloc(const dca_problem* problem, int32_t n
   w.vs[0] = (int32_t*)(base + kOffSpin);
   w.N[0][0] = (double*)(base + kOffN0);
   w.N[0][1] = (double*)(base + kOffN1);
-  w.Lrow[0] = (double*)(base + kOffScr0);
-  w.Lrow[1] = (double*)(base + kOffScr1);
+  w.gjX[0] = (double*)(base + kOffScr0);
+  w.gjX[1] = (double*)(base + kOffScr1);
   int32_t* d_sgn = (int32_t*)(base + kOffSign);
 
   std::vector<int32_t> site(n), s(n);

@@ -25,7 +25,8 @@
 // Bound by FP64 issue (a warp-wide FP64 instruction holds its SM sub-partition's
 // unit for 64 cycles): n^3 multiply-adds on 2 C per cycle.  A rank-1 pass over
 // the matrix per column instead made it wait on L2 and on two cluster barriers
-// a column: two matrices of order 500 (dca_fresh_N) 12.8 -> 5.6 ms a call.
+// a column: two matrices of order 500 (dca_fresh_N) 12.8 -> 4.33 ms a call on two
+// clusters, and 3.21 with the updates on the whole device (below).
 #include <cooperative_groups.h>
 
 #include <cstdint>
@@ -88,7 +89,7 @@ __device__ void gj_matrix(const Config& cfg, int mode, int mat, int* sgn_out, cg
   WalkerDev& w = cfg.W[wi];
   const int n = w.n, ld = w.cap;
   double* A = (cfg.prec == PREC_MIXED) ? w.Ascr[sp] : (double*)w.N[mode == 1 ? w.parity ^ 1 : w.parity][sp];
-  double* X = w.Lrow[sp];  // scratch [16][n]: rows J of the other columns; row buffers of the last step
+  double* X = w.gjX[sp];  // scratch [16][n]: rows J of the other columns; row buffers of the last step
   extern __shared__ __align__(16) unsigned char gj_smem[];
   // rp [n]: original row now at each position; in shared memory with panels of
   // 16, else one copy per block behind the first 8 rows of the scratch
@@ -415,7 +416,7 @@ __global__ void __launch_bounds__(256) k_gj_update(Config cfg, int c0, const int
         const int sp = s & 1, n = w.n, ld = w.cap, b = min(GW_B, n - c0), cblocks = (n + GW_C - 1) / GW_C;
         const int i0 = (item / cblocks) * GW_R, k0 = (item % cblocks) * GW_C, col = k0 + k;
         double* A = cfg.prec == PREC_MIXED ? w.Ascr[sp] : (double*)w.N[w.parity][sp];
-        const double* X = w.Lrow[sp];
+        const double* X = w.gjX[sp];
         const double* P = X + 16 * (size_t)n;
         __syncthreads();  // the previous item is done with the shared tiles
         for (int e = tid; e < GW_B * GW_C; e += 256) {
@@ -446,7 +447,7 @@ __global__ void __launch_bounds__(256) k_gj_finish(Config cfg, const int* sgn) {
   const int mat = blockIdx.y, sp = mat & 1, i = blockIdx.x;
   const WalkerDev& w = cfg.W[mat >> 1];
   if (i >= w.n || sgn[mat] == 0) return;
-  const int* rp = reinterpret_cast<const int*>(w.Lrow[sp] + 32 * (size_t)w.n);
+  const int* rp = reinterpret_cast<const int*>(w.gjX[sp] + 32 * (size_t)w.n);
   double* A = (cfg.prec == PREC_MIXED ? w.Ascr[sp] : (double*)w.N[w.parity][sp]) + (size_t)i * w.cap;
   for (int k = threadIdx.x; k < w.n; k += blockDim.x) row[k] = A[k];
   __syncthreads();

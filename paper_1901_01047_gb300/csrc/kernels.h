@@ -12,14 +12,14 @@ namespace dca {
 enum Group : int {
   GROUP_PROPOSE = 0,         // k_begin
   GROUP_EXTEND = 1,          // k_cand_zero, k_ext64, k_cc64 (mixed: k_ext_g, k_ext_x, k_cand_cc)
-  GROUP_METROPOLIS = 2,      // k_metropolis
+  GROUP_METROPOLIS = 2,      // k_metropolis64 (double-float Gamma: k_metropolis)
   GROUP_UPDATE = 3,          // the rank-l update of N
   GROUP_MEASURE = 4,         // k_meas_*
-  GROUP_RECOMPUTE = 5,       // k_gj_cluster
+  GROUP_RECOMPUTE = 5,       // k_gj_cluster (mixed: k_oz_a, k_oz_slice_n, k_refine_oz, k_correct_tc or k_refine_*)
   GROUP_UPDATE_PRE = 6,      // k_upd_factors (tcgen05 path) or k_upd_lp_rr
   GROUP_UPDATE_POST = 7,     // k_upd_border (tcgen05 path), k_window_end, k_compact_N, k_compact_end
   GROUP_RECOMPUTE_PRE = 8,   // k_build_A
-  GROUP_RECOMPUTE_POST = 9,  // (k_store_fp32), k_recompute_drift, k_recompute_adopt
+  GROUP_RECOMPUTE_POST = 9,  // k_refine_adopt or (k_store_fp32), k_recompute_drift; k_recompute_adopt
   N_GROUPS = 10,
 };
 
@@ -57,7 +57,7 @@ void launch_init(const Config& cfg, int n0, int max_cap, int* d_sgn, cudaStream_
 void launch_rebuild(const Config& cfg, int max_n, int* d_sgn, cudaStream_t st);
 void launch_fresh_inverse(const Config& cfg, int max_n, int* d_sgn, cudaStream_t st, bool wide = false);
 // The inverse spread over the whole device, for matrices of order n that all
-// walkers share (dca_fresh_N) with gj_wide_scratch(n) bytes behind Lrow; false
+// walkers share (dca_fresh_N) with gj_wide_scratch(n) bytes behind gjX; false
 // (nothing launched) where the order or the device is better served by launch_gj.
 size_t gj_wide_scratch(int n);
 bool launch_gj_wide(const Config& cfg, int n, int* d_sgn, cudaStream_t st);

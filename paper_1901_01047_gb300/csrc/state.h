@@ -32,6 +32,7 @@
 namespace dca {
 
 constexpr int KS_MAX = 128;     // largest submatrix size (App. B default is 128)
+constexpr int GJ_X_ROWS = 16;   // rows of n doubles that the Gauss-Jordan inverse of order n keeps as scratch
 
 enum : int32_t {
   ST_OK = 0,
@@ -152,7 +153,7 @@ struct WalkerDev {
   int64_t n_neglected;       // proposals rejected by the neglect rule
   int32_t* acc_slot;         // [KS_MAX] candidate slot of the m-th accepted insertion
   int32_t* acc_p;            // [KS_MAX] its position in P
-  double* Lrow[2];           // [spin][cap][KS_MAX] rows of L at extended row index
+  double* gjX[2];            // [spin][GJ_X_ROWS][n] scratch of the Gauss-Jordan inverse
   double* Lp[2];             // [spin][cap][KS_MAX] rows of L Binv at extended row index
   void* Rr[2];               // [spin][KS_MAX][cap] rows of R = N_ext[P, 0:n) (arithmetic type)
   float* Aop[2];             // [spin][hi, lo][cap][KS_MAX] split L' rows (tensor-core update)

@@ -439,7 +439,7 @@ extern "C" DCA_API int dca_walker_create(const dca_walker_params* prm, void* cud
       pieces.push_back({(void**)&w.Ub[sp], sizeof(double) * KS * C});
       pieces.push_back({(void**)&w.Binv[sp], sizeof(double) * KS * KS});
       pieces.push_back({(void**)&w.aP[sp], sizeof(double) * KS});
-      pieces.push_back({(void**)&w.Lrow[sp], sizeof(double) * KS * C});
+      pieces.push_back({(void**)&w.gjX[sp], sizeof(double) * dca::GJ_X_ROWS * C});
       pieces.push_back({(void**)&w.Lp[sp], sizeof(double) * KS * C});
       pieces.push_back({(void**)&w.Rr[sp], esz * KS * C});
       if (alloc_tc) {
@@ -1680,8 +1680,8 @@ extern "C" DCA_API int dca_fresh_N(const dca_problem* problem, int32_t n, const 
   w.vs[0] = d_s;
   w.N[0][0] = d_N[0];
   w.N[0][1] = d_N[1];
-  w.Lrow[0] = d_scr[0];
-  w.Lrow[1] = d_scr[1];
+  w.gjX[0] = d_scr[0];
+  w.gjX[1] = d_scr[1];
   std::vector<int32_t> site(n), s(n);
   std::vector<double> tau(n);
   for (int i = 0; i < n; ++i) {
