@@ -79,8 +79,9 @@ extern "C" {
  *           the same trajectory are 1e-6..1e-4 relative, growing with the conditioning
  *           of N^-1 and with the updates since the last recompute; with N recomputed
  *           before every measurement (recompute_at_measure) the accumulated G is within
- *           about 3e-7 (condition numbers up to 1e5), 0.3e-6 to 1.4e-5 at 16 sites and
- *           beta = 16 (1e6 to 4e8), as with N from the Gauss-Jordan inverse.
+ *           about 3e-7 (condition numbers up to 1e5), 0.3e-6 to 1e-5 at 16 sites and
+ *           beta = 16 (1e6 to 4e7), as with N from the Gauss-Jordan inverse
+ *           (DCA_RECOMPUTE_GJ, which also serves chains whose R reaches 0.03 and more).
  *   TF32:   as MIXED with one TF32 product per K step instead of three (the
  *           tensor-core kernels only); about 11 bits per product. */
 #define DCA_PREC_FP64 0
@@ -203,12 +204,12 @@ typedef struct {
  * from scratch in FP64 for the current configuration):
  *   AUTO:      DCA_PREC_FP64 inverts it by Gauss-Jordan with partial
  *              pivoting; the mixed paths apply one Newton step
- *              N <- N + N (I - A N) whose residual I - A N is formed on the
- *              tensor cores from exponent-aligned 9-bit digit planes of A (5)
+ *              N <- N + N R (+ N R^2 where max |R| is 2.5e-4 or more), whose
+ *              residual R = I - A N is formed on the tensor cores from exponent-aligned 9-bit digit planes of A (5)
  *              and N (4), the leading plane products summed exactly (Ozaki
  *              et al., Numer. Algorithms 59, 2012): about 2^-40 of the row /
  *              column maxima, so the step brings the FP32 N back to its
- *              rounding level.  Needs 18 cap^2 bytes per spin and walker.
+ *              rounding level unless R nears one.  Needs 18 cap^2 bytes per spin and walker.
  *   GJ:        Gauss-Jordan on both paths.
  *   NEWTON_DF: the mixed paths' Newton step with the residual in double-float
  *              arithmetic on the CUDA cores (about 2^-44 of sum |A| |N|). */

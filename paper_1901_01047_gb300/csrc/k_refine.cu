@@ -9,19 +9,19 @@
 // FP32 rounding level.  After a window close to singular R can be far larger,
 // and rows of N enter G with e^V - 1 (1.5e3 at 16 sites, beta = 16): on one of 100
 // chains there (order 590, max |R| = 0.03, condition number 4e8) one step left
-// 1.5e-4 of G, another build 2.7e-3.  So where max |R| of a walker-spin is 2.5e-4
+// 1.5e-4 of G, rounded otherwise 2.7e-3.  So where max |R| of a walker-spin is 2.5e-4
 // or more, the next term of N1 = N0 (I + R + R^2 + ...) follows, (N0 R) R from the
 // first one, by the same kernel; it is added if it is no more than half the first.
-// That chain's G: 1.4e-5 and 6.6e-5 in two builds (its rounding decides how large R
-// gets), with the Gauss-Jordan inverse 7e-6.  The idle launch is lost in the noise of
-// a pass, with what it computes a pass takes 0.3 to 1.6 % more.  Where R is of order
+// That chain's G: 1.4e-5 to 6.6e-5 (the rounding before decides how large R gets),
+// with the Gauss-Jordan inverse 7e-6.  The idle launch is lost in the noise of a
+// pass, with what it computes a pass takes 0.3 to 1.6 % more.  Where R is of order
 // one, as after a random start far from equilibrium, no Newton step helps: such
 // chains are for DCA_RECOMPUTE_GJ.
 //
 // Both products are tiled GEMMs on a persistent grid over (walker-spin, 64 x 64
 // output tile), so one walker's recompute spreads over every SM.  The residual is
-// the whole cost; it runs on the FP32 pipes in double-float arithmetic because GB300's FP64 units
-// issue ~2 FMA per clock per SM against 128 FP32 operations.
+// the whole cost; it runs on the FP32 pipes in double-float arithmetic because GB300's
+// FP64 units issue ~2 FMA per clock per SM against 128 FP32 operations.
 //
 // Buffers (the recompute follows a compaction, all n rows live):
 //   A   Ascr[sp] (FP32 pairs)    -> R  into N[parity ^ 1][sp] (FP32; from the digit planes R^T, see k_refine_tc.cu)
