@@ -205,11 +205,12 @@ typedef struct {
  *   AUTO:      DCA_PREC_FP64 inverts it by Gauss-Jordan with partial
  *              pivoting; the mixed paths apply one Newton step
  *              N <- N + N R (+ N R^2 where max |R| is 2.5e-4 or more), whose
- *              residual R = I - A N is formed on the tensor cores from exponent-aligned 9-bit digit planes of A (5)
- *              and N (4), the leading plane products summed exactly (Ozaki
- *              et al., Numer. Algorithms 59, 2012): about 2^-40 of the row /
- *              column maxima, so the step brings the FP32 N back to its
- *              rounding level unless R nears one.  Needs 18 cap^2 bytes per spin and walker.
+ *              residual R = I - A N is formed on the tensor cores from
+ *              exponent-aligned 9-bit digit planes of A (5) and N (4), the
+ *              leading plane products summed exactly (Ozaki et al., Numer.
+ *              Algorithms 59, 2012): about 2^-40 of the row / column maxima,
+ *              so the step brings the FP32 N back to its rounding level
+ *              unless R nears one.  Needs 18 cap^2 bytes per spin and walker.
  *   GJ:        Gauss-Jordan on both paths.
  *   NEWTON_DF: the mixed paths' Newton step with the residual in double-float
  *              arithmetic on the CUDA cores (about 2^-44 of sum |A| |N|). */
